@@ -46,9 +46,8 @@ typedef enum {
     SIBFA_E_NOT_CONVERGED = -3,  /* PCG hit max_iter above the tolerance        */
     SIBFA_E_CUTOFF = -4,         /* rc + 2 * site extent exceeds half the box   */
     SIBFA_E_CT_DENOM = -5,       /* a charge-transfer denominator dE <= 0       */
-    SIBFA_E_TIMEOUT = -6,        /* reserved: no kernel of this library waits on
-                                    another (grid-wide steps use cooperative
-                                    launches), so no call returns it             */
+    SIBFA_E_TIMEOUT = -6,        /* a wait between the blocks of the polarization
+                                    solve's cooperative kernel ran out (seconds)  */
     SIBFA_E_CUDA = -7,           /* a CUDA / cuFFT call failed                  */
     SIBFA_E_BUSY = -8,           /* admission refused (serving)                 */
     SIBFA_E_NEIGHBOR = -9        /* neighbour list overflow                     */
@@ -181,11 +180,12 @@ typedef struct sibfa_ctx sibfa_ctx;
 
 /* Create a context: validates sizes, copies the topology, builds the SPME
  * influence function and FFT plans, allocates all device state.  *out is
- * NULL on failure.  The PCG loop normally runs on the device as a CUDA graph
- * with a conditional while-node; with the environment variable
- * SIBFA_PCG_HOST_LOOP=1 at creation it is driven from the host instead (one
- * launch per kernel and iteration, same arithmetic), which kernel profilers
- * can follow.  The context tunes the schedule of its short-range kernels
+ * NULL on failure.  The PCG loop runs on the device: for one system of up to
+ * some 1700 waters, on a grid whose axes are products of 2, 3 and 5, as one
+ * cooperative kernel, otherwise as a CUDA graph with a conditional
+ * while-node.  With the environment variable SIBFA_PCG_HOST_LOOP=1 at
+ * creation it is driven from the host instead (one launch per kernel and
+ * iteration), which kernel profilers can follow.  The context tunes the schedule of its short-range kernels
  * (resident blocks per SM, and whether they finish before the polarization
  * solve; see sibfa_tuned_schedule) over its first full evaluations outside
  * sibfa_minimize by timing them and then keeps the fastest; the choice

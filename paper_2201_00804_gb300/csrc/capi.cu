@@ -13,6 +13,7 @@
 
 #include "sibfa_internal.cuh"
 #include "pcg_guess.cuh"
+#include "pcg_loop.cuh"
 #include "server_internal.h"
 
 using namespace sibfa;
@@ -64,6 +65,7 @@ struct sibfa_ctx {
     int pcg_graph_state = 0;     // 0 untried, 1 in use, -1 unavailable (host loop)
     uint64_t pcg_iter_launches = 0;
     uint64_t pcg_graph_solves = 0;   // graph solves whose iteration count is not yet folded into launches
+    LoopPlan loop;               // solve in one kernel (ncta > 0)
     bool capturing = false;
     int prec = SIBFA_PREC_MIXED;
     DevState<float> df{};
@@ -652,14 +654,21 @@ MuGuess mu_guess(const sibfa_ctx *ctx, bool full) {
     return g;
 }
 
-// Store the converged dipoles of a full evaluation (stream-ordered after the solve).
-sibfa_status push_mu(sibfa_ctx *ctx, const double *mu, bool full) {
-    if (!full || ctx->opts.warm_start < 2) return SIBFA_OK;
-    const size_t stride = (size_t)ctx->capacity * 9;
-    CK(cudaMemcpyAsync(ctx->mu_hist + (size_t)ctx->hist_head * stride, mu, (size_t)ctx->M * 9 * sizeof(double),
-                       cudaMemcpyDeviceToDevice, ctx->s));
+// Where the converged dipoles of a full evaluation are stored (null: nowhere).
+double *mu_slot(sibfa_ctx *ctx, bool full) {
+    if (!full || ctx->opts.warm_start < 2) return nullptr;
+    return ctx->mu_hist + (size_t)ctx->hist_head * ctx->capacity * 9;
+}
+void mu_pushed(sibfa_ctx *ctx) {
     ctx->hist_head = (ctx->hist_head + 1) % ctx->opts.warm_start;
     ctx->hist_n = std::min(ctx->hist_n + 1, ctx->opts.warm_start);
+}
+// Store them (stream-ordered after the solve).
+sibfa_status push_mu(sibfa_ctx *ctx, const double *mu, bool full) {
+    double *slot = mu_slot(ctx, full);
+    if (!slot) return SIBFA_OK;
+    CK(cudaMemcpyAsync(slot, mu, (size_t)ctx->M * 9 * sizeof(double), cudaMemcpyDeviceToDevice, ctx->s));
+    mu_pushed(ctx);
     return SIBFA_OK;
 }
 
@@ -668,6 +677,20 @@ sibfa_status solve(sibfa_ctx *ctx, DevState<R> &d, double tol, Launch L, bool fu
     const KParams &p = ctx->kp;
     const int warm = (ctx->opts.warm_start && ctx->have_mu) ? 1 : 0;
     const MuGuess g = mu_guess(ctx, full);
+    if (ctx->loop.ncta > 0) {
+        // serial profiling: the real-space product alone (its result is not used)
+        if (ctx->serial) {
+            CK(cudaMemsetAsync(d.flags + 1, 0, sizeof(int), ctx->s));
+            Phase ph(ctx, "real_tmu");
+            launch_real_tmu(p, d, d.efp, L);
+        }
+        double *push = mu_slot(ctx, full);
+        CK(launch_pcg_loop(p, d, ctx->loop, g, warm, push, L));
+        if (push) mu_pushed(ctx);
+        CK(cudaMemcpyAsync(ctx->h_scal, d.scal, 16 * sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
+        ctx->have_mu = true;
+        return SIBFA_OK;
+    }
     if (g.n > 0) launch_pcg_init_guess(p, d, g, L);
     else launch_pcg_init(p, d, warm, L);
     sibfa_status st = matvec(ctx, d, d.mu, L);
@@ -745,7 +768,8 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
         // neighbour list and the real-space pair kernels
         if ((st = fork_rec(ctx))) return st;
         Phase ph(ctx, "spme_perm", ctx->s2);
-        CK(cudaMemsetAsync(d.grid, 0, ng * sizeof(R), ctx->s2));
+        // the second grid takes the solve kernel's spreads
+        CK(cudaMemsetAsync(d.grid, 0, (ctx->loop.ncta ? 2 : 1) * ng * sizeof(R), ctx->s2));
         launch_spread(p, d, SPREAD_PERM, nullptr, d.grid, L2);
         if ((st = fft(ctx, d, true, 1))) return st;
         if (p.vir) launch_convolve_vir(p, d, 0, L2);
@@ -855,6 +879,10 @@ sibfa_status check_flags(sibfa_ctx *ctx, int flags) {
     if (flags & F_NEIGHBOR) {
         ctx->err = "neighbour list overflow";
         return SIBFA_E_NEIGHBOR;
+    }
+    if (flags & F_TIMEOUT) {
+        ctx->err = "a wait between blocks of the polarization solve ran out";
+        return SIBFA_E_TIMEOUT;
     }
     if (flags & F_CTDEN) {
         ctx->err = "charge-transfer denominator ae + V - ah <= 0";
@@ -1029,6 +1057,33 @@ sibfa_status create_impl(sibfa_ctx *ctx, const sibfa_topology *topo) {
         CK(cudaMemcpyAsync(d.cl_of, of.data(), M * sizeof(int), cudaMemcpyHostToDevice, ctx->s));
     }
     CK(cudaStreamSynchronize(ctx->s));
+    // the solve in one kernel: one system whose grid axes factor into small
+    // primes (cluster batches stop on each cluster's residual; the host loop
+    // is for profilers)
+    if (ctx->kp.n_cl == 1 && ctx->pcg_graph_state != -1) {
+        int dev = 0, n_sm = 0;
+        CK(cudaGetDevice(&dev));
+        CK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+        LoopPlan lp;
+        loop_plan<R>(lp, M, ctx->opts.periodic, ctx->kp.K, ctx->kp.tls, n_sm);
+        if (lp.ncta > 0) {
+            AL(lp.part, 3 * lp.ncta);
+            R *vec = nullptr;
+            AL(vec, (size_t)M * 12);
+            lp.vec = vec;
+            lp.maxit = ctx->opts.pcg_max_iter > 0 ? ctx->opts.pcg_max_iter : 200;
+            if (ctx->opts.periodic) {
+                const std::vector<double> t = loop_twiddles(ctx->kp.K);
+                const std::vector<R> tr(t.begin(), t.end());
+                R *tw = nullptr;
+                AL(tw, tr.size());
+                CK(cudaMemcpyAsync(tw, tr.data(), tr.size() * sizeof(R), cudaMemcpyHostToDevice, ctx->s));
+                CK(cudaStreamSynchronize(ctx->s));   // the host table is freed on return
+                lp.tw = tw;
+            }
+            ctx->loop = lp;
+        }
+    }
     if (ctx->opts.periodic) {
         Launch L{ctx->s, &ctx->launches};
         launch_influence(ctx->kp, d.infl, L);
@@ -1540,6 +1595,7 @@ sibfa_status ctx_set_batch(sibfa_ctx *ctx, int M, int n_cl, const int *cluster_s
     if (ctx->pcg_exec) cudaGraphExecDestroy(ctx->pcg_exec);
     ctx->pcg_exec = nullptr;
     ctx->pcg_graph_state = -1;
+    ctx->loop.ncta = 0;   // laid out for the first size
     return SIBFA_OK;
 }
 

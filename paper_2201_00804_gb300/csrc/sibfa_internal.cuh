@@ -22,7 +22,7 @@ constexpr int ORDER = 5;       // B-spline order of the SPME
 constexpr int VK_BLOCKS = 304;  // blocks of the virial convolution (fixed, so its partial sums have a fixed layout)
 
 // error flags (bitwise, device side)
-enum { F_CUTOFF = 1, F_NEIGHBOR = 2, F_CTDEN = 4, F_NAN = 8, F_NOCONV = 16 };
+enum { F_CUTOFF = 1, F_NEIGHBOR = 2, F_CTDEN = 4, F_NAN = 8, F_NOCONV = 16, F_TIMEOUT = 32 };
 
 // Scalars read inside pair loops, rounded once per precision on the host so
 // that the FP32 kernels do no FP64 conversion in their loops.
