@@ -7,14 +7,22 @@
 // visited from both sides.  Pair arithmetic runs in R (float in the mixed
 // path, double in the FP64 path); per-lane partial sums are reduced across
 // the warp in double.
-#include "sibfa_internal.cuh"
+#include <type_traits>
+
+#include "pair_terms.cuh"
 
 namespace sibfa {
+
 
 template <typename R>
 __device__ inline void symadd(Sym<R> &a, const Sym<R> &b, R s) {
     a.xx += s * b.xx; a.yy += s * b.yy; a.zz += s * b.zz;
     a.xy += s * b.xy; a.xz += s * b.xz; a.yz += s * b.yz;
+}
+template <typename R>
+__device__ __forceinline__ void symacc(Sym<R> &a, const Sym<R> &b) {
+    a.xx += b.xx; a.yy += b.yy; a.zz += b.zz;
+    a.xy += b.xy; a.xz += b.xz; a.yz += b.yz;
 }
 
 // ---------------------------------------------------------------------------
@@ -26,6 +34,12 @@ __device__ inline void symadd(Sym<R> &a, const Sym<R> &b, R s) {
 // lanes stay busy whatever the cutoff rejects; the tail is flushed at the
 // end.  Atom and midpoint sources go to separate queues because only atom
 // sources carry a valence (penetration), which keeps every round uniform.
+//
+// The target kernels below run one target site per block of one warp.  They
+// are bound by issue and by the latency of each round's source loads, so what
+// counts is warps per SM: blocks of one warp take any register count that
+// divides the file (112 registers, 18 warps, against 15 in blocks of five),
+// and a molecule's heavy targets (atoms) do not hold up its light ones.
 // ---------------------------------------------------------------------------
 constexpr int QCAP_A = 128;   // >= 31 carried + 3 atom sites x 32 new entries
 constexpr int QCAP_M = 96;    // >= 31 carried + 2 midpoints x 32 new entries
@@ -34,8 +48,8 @@ template <typename R, int CAP = QCAP_A + QCAP_M>
 struct PairQueue {
     int js[CAP];   // j * 8 + s
     R rx[CAP], ry[CAP], rz[CAP];
-    __device__ inline void put(int e, int j, int s, V3<R> r) {
-        js[e] = j * 8 + s;
+    __device__ inline void put(int e, int js_, V3<R> r) {
+        js[e] = js_;
         rx[e] = r.x;
         ry[e] = r.y;
         rz[e] = r.z;
@@ -45,15 +59,23 @@ struct PairQueue {
 
 // ---------------------------------------------------------------------------
 // Permanent electrostatics + penetration (Eq. 2), Thole-damped permanent
-// field on the polarizable atoms, potential on the lone pairs.
-// Warps 0..4: target site w of molecule i.  Warps 5, 6: target lone pair.
+// field on the polarizable atoms.
 // ---------------------------------------------------------------------------
 template <typename R>
 struct PermAcc {
-    Acc<R> Ue, Up, Vl;
+    Acc<R> Ue, Up;
     V3<R> gr, gm, ef;
-    Sym<R> gt;
-    R W[9];   // virial (VIR kernels only)
+    Sym<R> gt;   // three times the quadrupole sensitivity
+    R W[9];      // virial (VIR kernels only)
+};
+
+// A warp's target site
+template <typename R>
+struct PermT {
+    Mp<R> m;      // quadrupole / 3
+    V3<R> o;      // offset from O_i
+    R N, Q;       // valence; charge of molecule i (gas phase)
+    int w;        // site
 };
 
 // VIR: also accumulate the pair virial 1/2 g (x) x of the target's gradient g
@@ -83,191 +105,182 @@ struct PermAcc {
 // per target site and neighbour, and per source site on the O target's warp.
 // For gas-phase clusters this brings the FP32 multipole energy some 30x
 // closer to FP64 than summing the site-pair energies directly.
+//
+// ms: source multipole of site s_ (quadrupole / 3).  At a polarizable target
+// x, T2 and g1 return the pair's entry of the polarization matrix (field of a
+// dipole mu at x: T2 (mu.x) x + g1 mu).
 template <typename R, bool PER, bool ATOM_SRC, bool VIR>
-__device__ __forceinline__ void perm_pair(const KParams &p, const DevState<R> &d, int w, bool is_lp, V3<R> ot,
-                                          const Mp<R> &mt, R Nt_, R Qi, int js, V3<R> rv, size_t te,
-                                          PermAcc<R> &A) {
+__device__ __forceinline__ void perm_pair(const KParams &p, const PermT<R> &T, const Mp<R> &ms, int s_, V3<R> rv,
+                                          V3<R> osrc, PermAcc<R> &acc, R &g1, R &T2, V3<R> &x) {
     const Scal<R> &S = sc<R>(p);
-    const R third = R(1) / R(3);
-    const int j = js >> 3, s = js & 7;
-    V3<R> x, sv, osrc;
-    if (PER) {
-        x = ot - rv;
-    } else {
-        const R *os = d.off + (j * NP + s) * 3;
-        osrc = mk(__ldg(os), __ldg(os + 1), __ldg(os + 2));
-        sv = ot - osrc;
+    const bool atom = T.w < 3;
+    const R m1 = R(-1.0), two = R(2.0);
+    V3<R> sv;
+    if (PER) x = T.o - rv;
+    else {
+        sv = T.o - osrc;
         x = sv - rv;
     }
     const R r2 = dot(x, x);
-    const R rinv = rsqrt_(r2);
-    const R r = r2 * rinv;
-    const Mp<R> ms = load_mp_g(d.gmp + (j * NS + s) * GMP);
-    R g[6];
-    if (PER) g_erfc<R, 5>(r, rinv, S.alpha, g);
-    else g_bare<R, 5>(rinv, g);
-    if (is_lp) {
-        FieldTerms<R> f;
-        source_field<R, 1>(ms, x, g, f);
-        A.Vl.add(f.phi);
-        A.gr = A.gr + f.d1;
-        return;
-    }
-    FieldTerms<R> f;
-    source_field<R, 3>(ms, x, g, f);
+    const R rinv = rsqrt_<R>(r2);
+    const R r = r2 * rinv, r2i = rinv * rinv;
+    R B[6];
+    kernel_B<R, PER, 5>(r, rinv, r2i, S.alpha, B);
+    const Source<R> s(ms, x);
+    const Target<R> t(T.m, x);
+    const R pdt = symdd(s.th, t.th);
+    Field2<R> F;
+    const V3<R> gel = pair_grad(t, s, x, B, pdt, F);
     R U;
     if (PER) {
-        U = mt.q * f.phi + dot(mt.mu, f.d1) + third * symdd(mt.th, f.d2);
+        U = t.q * (s.q * B[0] + s.s * B[1] + s.w * B[2]) + dot(t.mu, F.d1) + F.Rr * t.w + two * dot(t.p, F.U) +
+            two * B[2] * pdt;
     } else {
-        const R a = rinv, a3 = a * a * a, a5 = a3 * a * a;
+        const R three = R(3.0);
+        const R a = rinv, a3 = a * r2i, a5 = a3 * r2i;
         // charge-charge, reference -D
-        const R RR = dot(rv, rv), b0 = rsqrt_(RR);
-        U = mt.q * ms.q * ((R(2) * dot(sv, rv) - dot(sv, sv)) * a * b0 / (r + RR * b0));
+        const R RR = dot(rv, rv), b0 = rsqrt_<R>(RR);
+        U = t.q * s.q * ((two * dot(sv, rv) - dot(sv, sv)) * a * b0 / (r + RR * b0));
         // target charge, reference O_i - x_s
-        const V3<R> y1 = R(-1) * (rv + osrc);
-        const R y1y1 = dot(y1, y1), b1 = rsqrt_(y1y1);
-        R B3, B5;
-        ref_diff35(-(R(2) * dot(y1, ot) + dot(ot, ot)), a, b1, r, y1y1 * b1, B3, B5);
-        const V3<R> Tso = symv(ms.th, ot), Tsy = symv(ms.th, y1);
-        const R mu_y1 = dot(ms.mu, y1), y1Ty1 = dot(y1, Tsy);
-        U += mt.q * (dot(ms.mu, ot) * a3 + mu_y1 * B3 + (dot(ot, Tso) + R(2) * dot(y1, Tso)) * a5 + y1Ty1 * B5);
-        if (w == 0) {   // sum over the target sites of q_t times the reference value: Q_i phi_s(y1)
+        const V3<R> y1 = m1 * (rv + osrc);
+        const R y1y1 = dot(y1, y1), b1 = rsqrt_<R>(y1y1);
+        R D3, D5;
+        ref_diff35(m1 * (two * dot(y1, T.o) + dot(T.o, T.o)), a, b1, r, y1y1 * b1, D3, D5);
+        const V3<R> Tso = symv(s.th, T.o), Tsy = symv(s.th, y1);
+        const R mu_y1 = dot(s.mu, y1), y1Ty1 = three * dot(y1, Tsy);
+        U += t.q * (dot(s.mu, T.o) * a3 + mu_y1 * D3 + three * (dot(T.o, Tso) + two * dot(y1, Tso)) * a5 + y1Ty1 * D5);
+        if (T.w == 0) {   // sum over the target sites of q_t times the reference value: Q_i phi_s(y1)
             const R b13 = b1 * b1 * b1;
-            U += Qi * (mu_y1 * b13 + y1Ty1 * b13 * b1 * b1);
+            U += T.Q * (mu_y1 * b13 + y1Ty1 * b13 * b1 * b1);
         }
         // source charge, reference x_t - O_j
-        const V3<R> y2 = ot - rv;
-        const R y2y2 = dot(y2, y2), b2 = rsqrt_(y2y2);
-        R C3, C5;
-        ref_diff35(R(2) * dot(y2, osrc) - dot(osrc, osrc), a, b2, r, y2y2 * b2, C3, C5);
-        const V3<R> Tto = symv(mt.th, osrc), Tty = symv(mt.th, y2);
-        U += ms.q * (dot(mt.mu, osrc) * a3 - dot(mt.mu, y2) * C3 + (dot(osrc, Tto) - R(2) * dot(y2, Tto)) * a5 +
-                     dot(y2, Tty) * C5);
+        const V3<R> y2 = T.o - rv;
+        const R y2y2 = dot(y2, y2), b2 = rsqrt_<R>(y2y2);
+        ref_diff35(two * dot(y2, osrc) - dot(osrc, osrc), a, b2, r, y2y2 * b2, D3, D5);
+        const V3<R> Tto = symv(t.th, osrc), Tty = symv(t.th, y2);
+        U += s.q * (dot(t.mu, osrc) * a3 - dot(t.mu, y2) * D3 + three * (dot(osrc, Tto) - two * dot(y2, Tto)) * a5 +
+                    three * dot(y2, Tty) * D5);
         // target dipole and quadrupole in the source dipole and quadrupole field
-        U += dot(mt.mu, f.d1_mp) + third * symdd(mt.th, f.d2_mp);
+        U += dot(t.mu, s.grad_mp(x, B[1], B[2], B[3])) + (s.s * B[3] + s.w * B[4]) * t.w + two * dot(t.p, F.U) +
+             two * B[2] * pdt;
     }
-    A.Ue.add(R(0.5) * U);
-    const V3<R> gel = target_grad(mt, ms, x, g, f);
-    A.gr = A.gr + gel;
-    V3<R> gv = gel;   // this pair's gradient (virial)
-    A.gm = A.gm + f.d1;
-    symadd(A.gt, f.d2, third);
+    acc.Ue.add(R(0.5) * U);
+    V3<R> g = gel;
+    acc.gm = acc.gm + F.d1;
+    symacc(acc.gt, F.d2);
     // ---- penetration: charge-charge*, charge-dipole*, charge-quadrupole*
     // Kernels exp(-b r)/r of the source (es) and target (et) valence; the
     // product kernel exp(-(b_s + b_t) r)/r of the N_t N_s term is es0 et0 r.
-    if (ATOM_SRC || Nt_ != R(0)) {
-        R pen = R(0), gq = R(0);
+    if (ATOM_SRC || atom) {
+        R pen = R(0.0), gq = R(0.0);   // gq: minus the coefficient of x from the charge terms
         R et[4];
-        const R xt_b = mulc(r, p.pen_b[w]);   // b_t r
-        if (Nt_ != R(0)) {
-            g_exp_x<R, 3>(xt_b, rinv, et);
-            const R c2 = ms.q * Nt_;            // q_s N_t exp(-b_t r)/r
-            pen += c2 * et[0];
-            gq += c2 * et[1];
+        const R xt = mulc(r, p.pen_b[T.w]);
+        if (atom) {
+            kernel_exp(xt, rinv, r2i, et);
+            const R c2 = s.q * T.N;            // q_s N_t exp(-b_t r)/r
+            pen = c2 * et[0];
+            gq = c2 * et[1];
         }
         if (ATOM_SRC) {
-            const R Ns = zsite<R>(p, s) - ms.q;
-            const R xs_b = mulc(r, p.pen_b[s]);   // b_s r
+            const R Ns = zsite<R>(p, s_) - ms.q, xs = mulc(r, p.pen_b[s_]);
             R es[4];
-            g_exp_x<R, 3>(xs_b, rinv, es);
-            const R c1 = mt.q * Ns;                // q_t N_s exp(-b_s r)/r
+            kernel_exp(xs, rinv, r2i, es);
+            const R c1 = t.q * Ns;             // q_t N_s exp(-b_s r)/r
             pen += c1 * es[0];
             gq += c1 * es[1];
-            if (Nt_ != R(0)) {                     // N_t N_s exp(-(b_t + b_s) r)/r
-                const R c3 = Nt_ * Ns;
-                const R ec = es[0] * et[0] * r;
-                pen += c3 * ec;
-                gq -= c3 * (xt_b + xs_b + R(1)) * ec * (rinv * rinv);
+            if (atom) {                      // N_t N_s exp(-(b_t + b_s) r)/r
+                const R ec = T.N * Ns * es[0] * et[0] * r;
+                pen += ec;
+                gq += (xt + xs + R(1.0)) * ec * r2i;
             }
-            // valence of s in the dipole/quadrupole potential of t
-            Mp<R> m0 = mt;
-            m0.q = R(0);
-            const V3<R> xs = -x;
-            FieldTerms<R> f3;
-            source_field<R, 1>(m0, xs, es, f3);
-            pen += Ns * f3.phi;
-            A.gr = A.gr - Ns * f3.d1;
-            if (VIR) gv = gv - Ns * f3.d1;
-            A.gm = A.gm + (-Ns * es[1]) * xs;
-            const R c = Ns * third * es[2];
-            A.gt.xx += c * xs.x * xs.x; A.gt.yy += c * xs.y * xs.y; A.gt.zz += c * xs.z * xs.z;
-            A.gt.xy += c * xs.x * xs.y; A.gt.xz += c * xs.x * xs.z; A.gt.yz += c * xs.y * xs.z;
+            // valence of s in the dipole/quadrupole potential of t, at -x
+            const R e2 = Ns * es[2], e1 = Ns * es[1];
+            pen += t.w * e2 - t.s * e1;
+            const R P = t.s * e2 - t.w * (Ns * es[3]), c = e2 + e2;
+            g = g + P * x + c * t.p - e1 * t.mu;
+            acc.gm = acc.gm - e1 * x;
+            const V3<R> ex = e2 * x;
+            acc.gt.xx += ex.x * x.x; acc.gt.yy += ex.y * x.y; acc.gt.zz += ex.z * x.z;
+            acc.gt.xy += ex.x * x.y; acc.gt.xz += ex.x * x.z; acc.gt.yz += ex.y * x.z;
         }
-        A.gr = A.gr + gq * x;
-        if (VIR) gv = gv + gq * x;
-        if (Nt_ != R(0)) {   // valence of t in the dipole/quadrupole potential of s
-            Mp<R> m0 = ms;
-            m0.q = R(0);
-            FieldTerms<R> f2;
-            source_field<R, 1>(m0, x, et, f2);
-            pen += Nt_ * f2.phi;
-            A.gr = A.gr + Nt_ * f2.d1;
-            if (VIR) gv = gv + Nt_ * f2.d1;
+        if (atom) {   // valence of t in the dipole/quadrupole potential of s
+            const R f1 = T.N * et[1], f2_ = T.N * et[2];
+            pen += s.s * f1 + s.w * f2_;
+            gq += s.s * f2_ + s.w * (T.N * et[3]);
+            const R c = f2_ + f2_;
+            g = g + f1 * s.mu + c * s.v;
         }
-        A.Up.add(R(0.5) * pen);
+        g = g - gq * x;
+        acc.Up.add(R(0.5) * pen);
     }
-    if (VIR) vir_add(A.W, gv, x, R(0.5));
-    // ---- Thole-damped permanent field on the polarizable atom (same base kernel g)
-    if (w < 3) {
-        R gtol[4];
-        g_thole_on<R, 3>(r, rinv, ainv3<R>(p, w, s), S.thole, PER, g, gtol);
-        FieldTerms<R> f4;
-        source_field<R, 1>(ms, x, gtol, f4);
-        A.ef = A.ef - f4.d1;
-        if (ATOM_SRC) {   // the same atom pair in the polarization matrix T
-            // the field of a dipole mu at x is g2 (mu.x) x + g1 mu = sgn(g2) (mu.y) y + g1 mu
-            // with y = sqrt|g2| x: four values and the sign of g2 in the index's top bit
-            const R sq = sqrt_(fabs(gtol[2]));
-            d.tl_j[te] = (j * 3 + s) | (gtol[2] < R(0) ? int(0x80000000u) : 0);
-            d.tl_x[te] = sq * x.x;
-            d.tl_y[te] = sq * x.y;
-            d.tl_z[te] = sq * x.z;
-            d.tl_g1[te] = gtol[1];
-        }
+    acc.gr = acc.gr + g;
+    if (VIR) vir_add(acc.W, g, x, R(0.5));
+    // ---- Thole-damped permanent field on the polarizable atom (same base kernel B)
+    if (atom) {
+        const R u = S.thole * r2 * r * ainv3<R>(p, T.w, s_);
+        const R e = exp_(m1 * u), c1 = e, c2 = e + u * e, c3 = c2 + R(0.6) * u * (u * e);
+        const R b1 = rinv * r2i, b2 = R(3.0) * b1 * r2i, b3 = R(5.0) * b2 * r2i;
+        const R T1 = B[1] - c1 * b1, T3 = B[3] - c3 * b3;
+        T2 = B[2] - c2 * b2;
+        acc.ef = acc.ef - s.grad(x, T1, T2, T3);
+        g1 = m1 * T1;
     }
 }
 
-// One block per molecule whose NW warps take the target points W0 ..
-// W0 + NW - 1: the five sites (W0 = 0) and, in a second launch on another
-// stream, the lone pairs (W0 = 5: potential and gradient).  POT: the atoms
-// O, H1, H2 as potential-only targets (potential and gradient, the acceptor
-// potentials of the original charge transfer).  Each warp stores
-// its energies, so the blocks need no barrier; the virial variant sums the
-// site warps' virials in a fixed order.
-// Site blocks: 3 resident per SM in periodic systems, 4 in the gas phase
-// (96 registers; measured faster there, slower with the Ewald kernels).
-template <typename R, bool PER, bool VIR, int W0, int NW, bool POT = false>
-__global__ void __launch_bounds__(32 * NW, NW == 5 ? (PER ? 3 : 4) : (NW == 3 ? 5 : 8))
+// Blocks per SM, FP32: periodic 18 (112 registers; 32,000 waters: 1728 us,
+// 1909 at 16, 1735 at 20, where registers spill, 1926 with the five sites in
+// one block), gas phase 17 (4096 clusters: 1409 us, 1423 at 18, 1444 before);
+// FP64 8 (216 waters: 274 us against 416 in one block).
+template <typename R, bool PER, bool VIR>
+__global__ void __launch_bounds__(VIR ? 32 * NS : 32,
+                                  VIR ? (sizeof(R) == 4 ? 3 : 2) : (sizeof(R) == 4 ? (PER ? 18 : 17) : 8))
     k_real_perm(KParams p, DevState<R> d) {
+    constexpr int NW = VIR ? NS : 1;   // warps a block: the virial variant sums the sites' in a fixed order
     __shared__ double s_w[VIR ? NW : 1][9];
     __shared__ PairQueue<R> qs[NW];
     static_assert(sizeof(PairQueue<R>) >= 15 * 33 * sizeof(R), "reduction buffer aliases the queue");
-    const int i = blockIdx.x;
-    const int wq = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int w = W0 + wq;   // target point
-    constexpr bool is_lp = W0 >= NS || POT;   // potential-only targets
+    const int wq = VIR ? threadIdx.x >> 5 : 0, lane = threadIdx.x & 31;
+    const int i = VIR ? blockIdx.x : blockIdx.x / NS;
+    const int w = VIR ? wq : blockIdx.x % NS;   // target site
     PairQueue<R> &q = qs[wq];
-    const V3<R> ot = my_pt(d, i, w);
-    Mp<R> mt{};
-    if (!is_lp) mt = load_mp(d.gmp + (i * NS + w) * GMP);
-    const R Nt = (!is_lp) ? zsite<R>(p, w) - mt.q * R(w < 3) : R(0);
-    const R Nt_ = (w < 3) ? Nt : R(0);
+    const Mp<R> mt = load_mp(d.gmp + (i * NS + w) * GMP);
+    R Qi = R(0);   // gas phase: charge of molecule i (remainders of the reference-difference energy, see perm_pair)
+    if (!PER)
+        for (int s = 0; s < NS; ++s) Qi += d.gmp[(i * NS + s) * GMP];
+    const PermT<R> T{scaled(mt, R(1.0 / 3.0)), my_pt(d, i, w), zsite<R>(p, w) - mt.q, Qi, w};
     const R rc2 = sc<R>(p).rc2;
     const size_t tbase = (size_t)(i * 3 + (w < 3 ? w : 0)) * p.tls;   // T-pair list of target atom w
 
-    PermAcc<R> A;
-    A.gr = mk(R(0), R(0), R(0));
-    A.gm = A.gr;
-    A.ef = A.gr;
-    A.gt = Sym<R>{};
+    PermAcc<R> acc;
+    acc.gr = mk(R(0), R(0), R(0));
+    acc.gm = acc.gr;
+    acc.ef = acc.gr;
+    acc.gt = Sym<R>{};
 #pragma unroll
-    for (int k = 0; k < 9; ++k) A.W[k] = R(0);
+    for (int k = 0; k < 9; ++k) acc.W[k] = R(0);
+
+    auto eval = [&](auto atom_src, int e, size_t te) {
+        constexpr bool AT = decltype(atom_src)::value;
+        const int js = q.js[e], j = js >> 3, s = js & 7;
+        const Mp<R> ms = scaled(load_mp_g(d.gmp + (j * NS + s) * GMP), R(1.0 / 3.0));
+        V3<R> os = mk(R(0), R(0), R(0)), x;
+        if (!PER) os = my_pt(d, j, s);
+        R g1 = R(0), T2 = R(0);
+        perm_pair<R, PER, AT, VIR>(p, T, ms, s, q.at(e), os, acc, g1, T2, x);
+        if (AT && w < 3) {
+            // the same atom pair in the polarization matrix T: the field of a
+            // dipole mu at x is T2 (mu.x) x + g1 mu = sgn(T2) (mu.y) y + g1 mu
+            // with y = sqrt|T2| x: four values and the sign in the index's top bit
+            const R sq = sqrt_(fabs(T2));
+            d.tl_j[te] = (j * 3 + s) | (T2 < R(0) ? int(0x80000000u) : 0);
+            d.tl_x[te] = sq * x.x;
+            d.tl_y[te] = sq * x.y;
+            d.tl_z[te] = sq * x.z;
+            d.tl_g1[te] = g1;
+        }
+    };
+
     int ha = 0, ta = 0, hm = 0, tm = 0;   // queue heads and tails (warp-uniform, monotone)
-    // gas phase: charge of molecule i (remainders of the reference-difference
-    // energy terms, see perm_pair)
-    R Qi = R(0);
-    if (!PER && !is_lp)
-        for (int s = 0; s < NS; ++s) Qi += d.gmp[(i * NS + s) * GMP];
     const int nn = d.nnbr[i];
     for (int base = 0;; base += 32) {
         const bool flush = base >= nn;   // list exhausted: evaluate what is left in the queues
@@ -283,20 +296,20 @@ __global__ void __launch_bounds__(32 * NW, NW == 5 ? (PER ? 3 : 4) : (NW == 3 ? 
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
                 rs[s] = dO + mk(__ldg(offj + s * 3), __ldg(offj + s * 3 + 1), __ldg(offj + s * 3 + 2));
-                const V3<R> x = ot - rs[s];
+                const V3<R> x = T.o - rs[s];
                 if (!PER || dot(x, x) < rc2) bits |= 1u << s;
                 if (!PER) rs[s] = dO;   // queued: the O-O displacement (see perm_pair)
             }
-            if (!PER && !is_lp) {
+            if (!PER) {
                 R Qj = R(0);
                 for (int s = 0; s < NS; ++s) Qj += d.gmp[(j * NS + s) * GMP];
                 // Q_j times the reference value of the target's terms: the
                 // charge-charge one (O target only) and the dipole/quadrupole ones
-                const V3<R> y2 = ot - dO;
+                const V3<R> y2 = T.o - dO;
                 const R b2 = rsqrt_(dot(y2, y2)), b23 = b2 * b2 * b2;
-                R rem = -dot(mt.mu, y2) * b23 + dot(y2, symv(mt.th, y2)) * b23 * b2 * b2;
+                R rem = R(3) * dot(y2, symv(T.m.th, y2)) * b23 * b2 * b2 - dot(T.m.mu, y2) * b23;
                 if (w == 0) rem += Qi * rsqrt_(dot(dO, dO));
-                A.Ue.add(R(0.5) * Qj * rem);
+                acc.Ue.add(R(0.5) * Qj * rem);
             }
         }
         int na, nm;
@@ -305,75 +318,45 @@ __global__ void __launch_bounds__(32 * NW, NW == 5 ? (PER ? 3 : 4) : (NW == 3 ? 
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
             if (!((bits >> s) & 1u)) continue;
-            int e;
-            if (s < 3) e = (ta + pa++) % QCAP_A;
-            else e = QCAP_A + (tm + pm++) % QCAP_M;
-            q.js[e] = j * 8 + s;
-            q.rx[e] = rs[s].x;
-            q.ry[e] = rs[s].y;
-            q.rz[e] = rs[s].z;
+            q.put(s < 3 ? (ta + pa++) % QCAP_A : QCAP_A + (tm + pm++) % QCAP_M, j * 8 + s, rs[s]);
         }
         ta += na;
         tm += nm;
         __syncwarp();
         while (ta - ha >= 32 || (flush && ta > ha)) {
-            if (lane < ta - ha) {
-                const int e = (ha + lane) % QCAP_A;
-                perm_pair<R, PER, true, VIR>(p, d, w, is_lp, ot, mt, Nt_, Qi, q.js[e], q.at(e), tbase + ha + lane,
-                                             A);
-            }
+            if (lane < ta - ha) eval(std::true_type{}, (ha + lane) % QCAP_A, tbase + ha + lane);
             ha += min(32, ta - ha);
         }
         while (tm - hm >= 32 || (flush && tm > hm)) {
-            if (lane < tm - hm) {
-                const int e = QCAP_A + (hm + lane) % QCAP_M;
-                perm_pair<R, PER, false, VIR>(p, d, w, is_lp, ot, mt, Nt_, Qi, q.js[e], q.at(e), 0, A);
-            }
+            if (lane < tm - hm) eval(std::false_type{}, QCAP_A + (hm + lane) % QCAP_M, 0);
             hm += min(32, tm - hm);
         }
         __syncwarp();
         if (flush) break;
     }
 
-    if (!POT && w < 3 && lane == 0) d.tl_n[i * 3 + w] = ta;
+    if (w < 3 && lane == 0) d.tl_n[i * 3 + w] = ta;
     const double ke = p.ke;
     R *buf = reinterpret_cast<R *>(&q);
-    if (POT) {
-        const double v = warp_sum_acc(A.Vl);
-        const R vals[3] = {A.gr.x, A.gr.y, A.gr.z};
-        const R t = warp_transpose_sum<R, 3>(vals, buf, lane);
-        if (lane < 3) d.dva[(i * 3 + w) * 3 + lane] += ke * double(t);
-        if (lane == 0) d.va[i * 3 + w] += ke * v;
-    } else if (is_lp) {
-        const int l = w - NS;
-        const double v = warp_sum_acc(A.Vl);
-        const R vals[3] = {A.gr.x, A.gr.y, A.gr.z};
-        const R t = warp_transpose_sum<R, 3>(vals, buf, lane);
-        if (lane < 3) d.dvlp[(i * 2 + l) * 3 + lane] += ke * double(t);
-        if (lane == 0) d.vlp[i * 2 + l] += ke * v;
-    } else {
-        const R vals[15] = {A.gr.x, A.gr.y, A.gr.z, A.gm.x, A.gm.y, A.gm.z, A.gt.xx, A.gt.yy, A.gt.zz,
-                            A.gt.xy, A.gt.xz, A.gt.yz, A.ef.x, A.ef.y, A.ef.z};
-        const R t = warp_transpose_sum<R, 15>(vals, buf, lane);
-        // one destination per lane, so the FP64 update is a single warp instruction
-        double *dst = nullptr;
-        if (lane < 3) dst = d.gpt + (i * NP + w) * 3 + lane;
-        else if (lane < 6) dst = d.gmu + (i * NS + w) * 3 + lane - 3;
-        else if (lane < 12) dst = d.gth + (i * NS + w) * 6 + lane - 6;
-        else if (lane < 15 && w < 3) dst = d.efield + i * 9 + w * 3 + lane - 12;
-        if (dst) *dst += (lane < 12 ? ke : 1.0) * double(t);
-        if (VIR) {
-            const R wv = warp_transpose_sum<R, 9>(A.W, buf, lane);
-            if (lane < 9) s_w[wq][lane] = double(wv);
-        }
-        // per-warp energies (summed over the five sites in a fixed order by k_pol_energy)
-        const double e0 = warp_sum_acc(A.Ue), e1 = warp_sum_acc(A.Up);
-        if (lane == 0) {
-            d.epw[(i * NS + w) * 2] = ke * e0;
-            d.epw[(i * NS + w) * 2 + 1] = ke * e1;
-        }
+    const R vals[15] = {acc.gr.x, acc.gr.y, acc.gr.z, acc.gm.x, acc.gm.y, acc.gm.z, acc.gt.xx, acc.gt.yy, acc.gt.zz,
+                        acc.gt.xy, acc.gt.xz, acc.gt.yz, acc.ef.x, acc.ef.y, acc.ef.z};
+    const R t = warp_transpose_sum<R, 15>(vals, buf, lane);
+    // one destination per lane, so the FP64 update is a single warp instruction
+    double *dst = nullptr;
+    if (lane < 3) dst = d.gpt + (i * NP + w) * 3 + lane;
+    else if (lane < 6) dst = d.gmu + (i * NS + w) * 3 + lane - 3;
+    else if (lane < 12) dst = d.gth + (i * NS + w) * 6 + lane - 6;
+    else if (lane < 15 && w < 3) dst = d.efield + i * 9 + w * 3 + lane - 12;
+    if (dst) *dst += (lane < 6 ? ke : (lane < 12 ? ke * (1.0 / 3.0) : 1.0)) * double(t);
+    // per-site energies (summed over the five sites in a fixed order by k_pol_energy)
+    const double e0 = warp_sum_acc(acc.Ue), e1 = warp_sum_acc(acc.Up);
+    if (lane == 0) {
+        d.epw[(i * NS + w) * 2] = ke * e0;
+        d.epw[(i * NS + w) * 2 + 1] = ke * e1;
     }
     if (VIR) {   // the site warps' virials in a fixed order
+        const R wv = warp_transpose_sum<R, 9>(acc.W, buf, lane);
+        if (lane < 9) s_w[wq][lane] = double(wv);
         __syncthreads();
         if (threadIdx.x < 9) {
             double v = 0;
@@ -386,15 +369,90 @@ __global__ void __launch_bounds__(32 * NW, NW == 5 ? (PER ? 3 : 4) : (NW == 3 ? 
 template <typename R>
 void launch_real_perm(const KParams &p, DevState<R> &d, Launch L) {
     if (p.vir) {
-        if (p.periodic) k_real_perm<R, true, true, 0, NS><<<p.M, 32 * NS, 0, L.s>>>(p, d);
-        else k_real_perm<R, false, true, 0, NS><<<p.M, 32 * NS, 0, L.s>>>(p, d);
-        count(L);
-        return;
+        if (p.periodic) k_real_perm<R, true, true><<<p.M, 32 * NS, 0, L.s>>>(p, d);
+        else k_real_perm<R, false, true><<<p.M, 32 * NS, 0, L.s>>>(p, d);
+    } else {
+        if (p.periodic) k_real_perm<R, true, false><<<p.M * NS, 32, 0, L.s>>>(p, d);
+        else k_real_perm<R, false, false><<<p.M * NS, 32, 0, L.s>>>(p, d);
     }
-    // the five sites in one block: as two launches (atoms, midpoints) the
-    // second launch's tail cost more than the uneven warps of one block
-    if (p.periodic) k_real_perm<R, true, false, 0, NS><<<p.M, 32 * NS, 0, L.s>>>(p, d);
-    else k_real_perm<R, false, false, 0, NS><<<p.M, 32 * NS, 0, L.s>>>(p, d);
+    count(L);
+}
+
+// Potential of the permanent multipoles and its gradient at the lone pairs
+// (ATOMS = false) or, for the original charge transfer, at O, H1 and H2: one
+// point per warp, the five source sites sharing one queue.
+constexpr int QCAP_P = 192;   // >= 31 carried + 5 sites x 32 new entries
+template <typename R, bool PER, bool ATOMS>
+__global__ void __launch_bounds__(128) k_potential(KParams p, DevState<R> d) {
+    constexpr int NPT = ATOMS ? 3 : 2;   // points a molecule
+    __shared__ PairQueue<R, QCAP_P> qs[4];
+    const int wq = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int a = blockIdx.x * 4 + wq, i = a / NPT;
+    if (i >= p.M) return;
+    PairQueue<R, QCAP_P> &q = qs[wq];
+    const V3<R> ot = my_pt(d, i, (ATOMS ? 0 : NS) + a % NPT);
+    const R rc2 = sc<R>(p).rc2, alpha = sc<R>(p).alpha;
+    Acc<R> V;
+    V3<R> gr = mk(R(0), R(0), R(0));
+    int h = 0, t = 0;
+    const int nn = d.nnbr[i];
+    for (int base = 0;; base += 32) {
+        const bool flush = base >= nn;
+        const int slot = base + lane;
+        unsigned bits = 0;
+        int j = 0;
+        V3<R> rs[NS];
+        if (slot < nn) {
+            j = d.nbr[i * MAXN + slot];
+            const R *dp = d.ndo + ((size_t)i * MAXN + slot) * 3;
+            const V3<R> dO = mk(dp[0], dp[1], dp[2]);
+            const R *offj = d.off + j * NP * 3;
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+                const V3<R> os = mk(__ldg(offj + s * 3), __ldg(offj + s * 3 + 1), __ldg(offj + s * 3 + 2));
+                // periodic: the source position; gas phase: the displacement
+                // formed as (target - source offset) - D, queued itself
+                rs[s] = PER ? dO + os : (ot - os) - dO;
+                const V3<R> x = ot - rs[s];
+                if (!PER || dot(x, x) < rc2) bits |= 1u << s;
+            }
+        }
+        int n;
+        int k = warp_excl_scan(__popc(bits), lane, n);
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+            if ((bits >> s) & 1u) q.put((t + k++) % QCAP_P, j * 8 + s, rs[s]);
+        t += n;
+        __syncwarp();
+        while (t - h >= 32 || (flush && t > h)) {
+            if (lane < t - h) {
+                const int e = (h + lane) % QCAP_P, js = q.js[e];
+                const V3<R> x = PER ? ot - q.at(e) : q.at(e);
+                const Source<R> src(scaled(load_mp_g(d.gmp + ((js >> 3) * NS + (js & 7)) * GMP), R(1.0 / 3.0)), x);
+                const R r2 = dot(x, x), rinv = rsqrt_(r2), r2i = rinv * rinv;
+                R B[4];
+                kernel_B<R, PER, 3>(r2 * rinv, rinv, r2i, alpha, B);
+                V.add(src.q * B[0] + src.s * B[1] + src.w * B[2]);
+                gr = gr + src.grad(x, B[1], B[2], B[3]);
+            }
+            h += min(32, t - h);
+        }
+        __syncwarp();
+        if (flush) break;
+    }
+    const double ke = p.ke;
+    const double v = warp_sum_acc(V);
+    const R vals[3] = {gr.x, gr.y, gr.z};
+    const R g = warp_transpose_sum<R, 3>(vals, reinterpret_cast<R *>(&q), lane);
+    if (lane < 3) (ATOMS ? d.dva : d.dvlp)[a * 3 + lane] += ke * double(g);
+    if (lane == 0) (ATOMS ? d.va : d.vlp)[a] += ke * v;
+}
+
+template <typename R, bool ATOMS>
+void launch_potential(const KParams &p, DevState<R> &d, Launch L) {
+    const unsigned nb = (unsigned)((p.M * (ATOMS ? 3 : 2) + 3) / 4);
+    if (p.periodic) k_potential<R, true, ATOMS><<<nb, 128, 0, L.s>>>(p, d);
+    else k_potential<R, false, ATOMS><<<nb, 128, 0, L.s>>>(p, d);
     count(L);
 }
 
@@ -402,14 +460,8 @@ void launch_real_perm(const KParams &p, DevState<R> &d, Launch L) {
 // space); with the original charge transfer also at the atoms O, H1, H2
 template <typename R>
 void launch_lp_potential(const KParams &p, DevState<R> &d, Launch L) {
-    if (p.periodic) k_real_perm<R, true, false, NS, 2><<<p.M, 64, 0, L.s>>>(p, d);
-    else k_real_perm<R, false, false, NS, 2><<<p.M, 64, 0, L.s>>>(p, d);
-    count(L);
-    if (p.ct_orig) {
-        if (p.periodic) k_real_perm<R, true, false, 0, 3, true><<<p.M, 96, 0, L.s>>>(p, d);
-        else k_real_perm<R, false, false, 0, 3, true><<<p.M, 96, 0, L.s>>>(p, d);
-        count(L);
-    }
+    launch_potential<R, false>(p, d, L);
+    if (p.ct_orig) launch_potential<R, true>(p, d, L);
 }
 
 // ---------------------------------------------------------------------------
@@ -506,12 +558,13 @@ __global__ void k_ct_prep(int M, int orig, DevState<R> d) {
 // the slots inside the cutoff (carrier-carrier distance) are queued in
 // shared memory and taken in full 32-lane rounds, each lane one molecule
 // pair with its 8 donor-acceptor items (i donating to j and j to i).
+template <typename R> constexpr int CW = sizeof(R) == 4 ? 4 : 1;   // molecules a block
 template <typename R, bool PER, bool VIR>
-__global__ void __launch_bounds__(128) k_ct(KParams p, DevState<R> d) {
-    __shared__ R red[4][23 * 33];
-    __shared__ int sq[4][64];
+__global__ void __launch_bounds__(32 * CW<R>) k_ct(KParams p, DevState<R> d) {
+    __shared__ R red[CW<R>][23 * 33];
+    __shared__ int sq[CW<R>][64];
     const int wq = threadIdx.x >> 5;
-    const int i = blockIdx.x * 4 + wq;
+    const int i = blockIdx.x * CW<R> + wq;
     const int lane = threadIdx.x & 31;
     if (i >= p.M) return;
     const R rc2 = sc<R>(p).rc2;
@@ -718,13 +771,13 @@ template <typename R>
 void launch_ct(const KParams &p, DevState<R> &d, Launch L) {
     k_ct_prep<R><<<(p.M + 127) / 128, 128, 0, L.s>>>(p.M, p.ct_orig, d);
     count(L);
-    const unsigned nb = (p.M + 3) / 4;
+    const unsigned nb = (p.M + CW<R> - 1) / CW<R>;
     if (p.vir) {
-        if (p.periodic) k_ct<R, true, true><<<nb, 128, 0, L.s>>>(p, d);
-        else k_ct<R, false, true><<<nb, 128, 0, L.s>>>(p, d);
+        if (p.periodic) k_ct<R, true, true><<<nb, 32 * CW<R>, 0, L.s>>>(p, d);
+        else k_ct<R, false, true><<<nb, 32 * CW<R>, 0, L.s>>>(p, d);
     } else {
-        if (p.periodic) k_ct<R, true, false><<<nb, 128, 0, L.s>>>(p, d);
-        else k_ct<R, false, false><<<nb, 128, 0, L.s>>>(p, d);
+        if (p.periodic) k_ct<R, true, false><<<nb, 32 * CW<R>, 0, L.s>>>(p, d);
+        else k_ct<R, false, false><<<nb, 32 * CW<R>, 0, L.s>>>(p, d);
     }
     count(L);
     if (p.ct_orig) {
@@ -799,98 +852,109 @@ constexpr int PQ_A = 128, PQ_M = 96, PQ_L = 96;
 template <typename R>
 struct PfAcc {
     V3<R> gr, gm;
-    Sym<R> gt;
-    R W[9];   // virial (VIR kernels only)
+    Sym<R> gt;   // three times the quadrupole sensitivity
+    R W[9];      // virial (VIR kernels only)
 };
 
 // VIR: also accumulate the pair virial g (x) x of the target's gradient g:
 // half of it for dipole and multipole sources (the partner adds the other
 // half), all of it for lambda charges (whose lone-pair side adds none).
+//
+// Each source is evaluated for what it has: the dipole and charge sources
+// carry no quadrupole, and at a polarizable target the source's permanent and
+// induced dipoles act on the target's induced dipole through one second
+// derivative, contracted as it is formed.  mt: quadrupole / 3.
 template <typename R, bool PER, int KIND, bool VIR>   // KIND 0: atom source, 1: midpoint source, 2: lambda charge
 __device__ __forceinline__ void polf_pair(const KParams &p, const DevState<R> &d, int w, V3<R> ot, const Mp<R> &mt,
                                           V3<R> mui, int js, V3<R> rs, PfAcc<R> &A) {
     const Scal<R> &S = sc<R>(p);
-    const R third = R(1) / R(3);
     const int j = js >> 3, s = js & 7;
     const V3<R> x = ot - rs;
     const R r2 = dot(x, x);
-    const R rinv = rsqrt_(r2), r = r2 * rinv;
+    const R rinv = rsqrt_(r2), r = r2 * rinv, r2i = rinv * rinv;
+    // charge source c at the target multipole: gradient and sensitivities
+    auto charge = [&](R c, const R *B, const Target<R> &t) {
+        const R P = -c * B[1], Q = c * B[2];
+        const V3<R> d1 = P * x;
+        A.gm = A.gm + d1;
+        const V3<R> qx = Q * x;
+        A.gt.xx += P + qx.x * x.x; A.gt.yy += P + qx.y * x.y; A.gt.zz += P + qx.z * x.z;
+        A.gt.xy += qx.x * x.y; A.gt.xz += qx.x * x.z; A.gt.yz += qx.y * x.z;
+        return (t.q * P + t.s * Q - t.w * c * B[3]) * x + P * t.mu + (Q + Q) * t.p;
+    };
     if (KIND == 2) {
-        R g[6];
-        if (PER) g_erfc<R, 5>(r, rinv, S.alpha, g);
-        else g_bare<R, 5>(rinv, g);
-        Mp<R> ms{};
-        ms.q = d.lamR[j * 2 + s];
-        FieldTerms<R> f;
-        source_field<R, 3>(ms, x, g, f);
-        const V3<R> gl = target_grad(mt, ms, x, g, f);
+        R B[4];
+        kernel_B<R, PER, 3>(r, rinv, r2i, S.alpha, B);
+        const Target<R> t(mt, x);
+        const V3<R> gl = charge(d.lamR[j * 2 + s], B, t);
         A.gr = A.gr + gl;
-        A.gm = A.gm + f.d1;
-        symadd(A.gt, f.d2, third);
         if (VIR) vir_add(A.W, gl, x, R(1));
         return;
     }
-    V3<R> gv = mk(R(0), R(0), R(0));   // this pair's gradient (virial)
-    R gb[5], g[6];
-    if (PER) g_erfc<R, 4>(r, rinv, S.alpha, gb);
-    else g_bare<R, 4>(rinv, gb);
-    g_thole_on<R, 4>(r, rinv, ainv3<R>(p, w, s), S.thole, PER, gb, g);
-    g[5] = R(0);
-    if (KIND == 0) {   // induced dipole of atom s of j at target site w
-        Mp<R> ms{};
+    R B[5], T[5];
+    kernel_B<R, PER, 4>(r, rinv, r2i, S.alpha, B);
+    {
+        const R u = S.thole * r2 * r * ainv3<R>(p, w, s);
+        const R e = exp_(-u), ue = u * e, u2e = u * ue;
+        const R c2 = e + ue, c3 = c2 + R(0.6) * u2e;
+        const R c4 = c2 + R(18.0 / 35.0) * u2e + R(9.0 / 35.0) * u * u2e;
+        const R b1 = rinv * r2i, b2 = R(3) * b1 * r2i, b3 = R(5) * b2 * r2i, b4 = R(7) * b3 * r2i;
+        T[1] = B[1] - e * b1;
+        T[2] = B[2] - c2 * b2;
+        T[3] = B[3] - c3 * b3;
+        T[4] = B[4] - c4 * b4;
+    }
+    V3<R> gv = mk(R(0), R(0), R(0));
+    V3<R> b = gv;
+    if (KIND == 0) {   // induced dipole b of atom s of j at target site w
         const R *mj = d.muR + j * 9 + s * 3;
-        ms.mu = mk(mj[0], mj[1], mj[2]);
-        FieldTerms<R> f;
-        source_field<R, 3>(ms, x, g, f);
-        const V3<R> gm = target_grad(mt, ms, x, g, f);
-        A.gr = A.gr + gm;
-        A.gm = A.gm + f.d1;
-        symadd(A.gt, f.d2, third);
+        b = mk(mj[0], mj[1], mj[2]);
+        const Target<R> t(mt, x);
+        const R sb = dot(b, x), P = -sb * T[2], Rr = sb * T[3];
+        const V3<R> U = (-T[2]) * b, W = T[3] * b;
+        const V3<R> d1 = P * x + T[1] * b;
+        const Sym<R> d2 = second(x, P, Rr * x + U, U);
+        A.gm = A.gm + d1;
+        symacc(A.gt, d2);
+        const V3<R> pu = symv(t.th, U);
+        const R c = R(2) * dot(t.p, W) - t.w * sb * T[4];
+        gv = t.q * d1 + symv(d2, t.mu) + (Rr + Rr) * t.p + R(2) * pu + c * x + t.w * W;
         if (p.ct_orig) {   // original charge transfer: dE/dV(a) as a charge on atom s of j, undamped
-            Mp<R> ml{};
-            ml.q = d.lamaR[j * 3 + s];
-            const R gl[6] = {gb[0], gb[1], gb[2], gb[3], gb[4], R(0)};
-            FieldTerms<R> fl;
-            source_field<R, 3>(ml, x, gl, fl);
-            A.gr = A.gr + target_grad(mt, ml, x, gl, fl);
-            A.gm = A.gm + fl.d1;
-            symadd(A.gt, fl.d2, third);
-        }
-        if (VIR) gv = gm;
-        // induced-induced, d/dr_a of mu_a . grad phi_b: for w < 3 the site
-        // damping polarizability is the atom's, so f is the atom-atom field
-        if (w < 3) {
-            const V3<R> gi = symv(f.d2, mui);
-            A.gr = A.gr + gi;
-            if (VIR) gv = gv + gi;
+            const V3<R> gl = charge(d.lamaR[j * 3 + s], B, t);
+            A.gr = A.gr + gl;
         }
     }
-    if (w < 3) {       // permanent multipoles of site s of j at polarizable atom w
-        const Mp<R> ms = load_mp_g(d.gmp + (j * NS + s) * GMP);
-        FieldTerms<R> f;
-        source_field<R, 2>(ms, x, g, f);
-        const V3<R> gp = symv(f.d2, mui);
-        A.gr = A.gr + gp;
-        if (VIR) gv = gv + gp;
+    if (w < 3) {
+        // permanent multipoles (and induced dipole) of site s of j at the
+        // induced dipole m of polarizable atom w: d/dx of m . grad phi
+        Mp<R> m = load_mp_g(d.gmp + (j * NS + s) * GMP);
+        if (KIND == 0) m.mu = m.mu + b;
+        const Source<R> q(scaled(m, R(1.0 / 3.0)), x);
+        const R P = -(q.q * T[1] + q.s * T[2] + q.w * T[3]);
+        const R Rr = q.q * T[2] + q.s * T[3] + q.w * T[4];
+        const V3<R> U = (-T[2]) * q.mu + (R(-2) * T[3]) * q.v;
+        const R xm = dot(x, mui);
+        gv = gv + P * mui + (Rr * xm + dot(U, mui)) * x + xm * U + (T[2] + T[2]) * symv(q.th, mui);
     }
+    A.gr = A.gr + gv;
     if (VIR) vir_add(A.W, gv, x, R(0.5));
 }
 
-// Target sites W0 .. W0 + NW - 1 of one molecule per block: the atoms and
-// the midpoints in two launches (the virial variant: all five in one block).
-// The gas-phase launches keep more blocks resident (fewer registers), which
-// measured faster there.
-template <typename R, bool PER, bool VIR, int W0, int NW>
-__global__ void __launch_bounds__(32 * NW, NW == 5 ? 3 : (NW == 3 ? (PER ? 5 : 6) : (PER ? 8 : 10))) k_real_polforce(KParams p,
-                                                                                          DevState<R> d) {
+// One target site of one molecule per block of one warp (the virial variant:
+// the five sites of a molecule in one block, summed in a fixed order).
+template <typename R, bool PER, bool VIR>
+__global__ void __launch_bounds__(VIR ? 32 * NS : 32, VIR ? 3 : (sizeof(R) == 4 ? 32 : 8))
+    k_real_polforce(KParams p, DevState<R> d) {
+    constexpr int NW = VIR ? NS : 1;
+    __shared__ double s_w[VIR ? NW : 1][9];
     __shared__ PairQueue<R, PQ_A + PQ_M + PQ_L> qs[NW];
     static_assert(sizeof(PairQueue<R, PQ_A + PQ_M + PQ_L>) >= 12 * 33 * sizeof(R), "reduction buffer");
-    const int i = blockIdx.x;
-    const int wq = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int w = W0 + wq;   // target site
+    const int wq = VIR ? threadIdx.x >> 5 : 0, lane = threadIdx.x & 31;
+    const int i = VIR ? blockIdx.x : blockIdx.x / NS;
+    const int w = VIR ? wq : blockIdx.x % NS;   // target site
     PairQueue<R, PQ_A + PQ_M + PQ_L> &q = qs[wq];
     const V3<R> ot = my_pt(d, i, w);
-    const Mp<R> mt = load_mp(d.gmp + (i * NS + w) * GMP);
+    const Mp<R> mt = scaled(load_mp(d.gmp + (i * NS + w) * GMP), R(1.0 / 3.0));
     V3<R> mui = mk(R(0), R(0), R(0));
     if (w < 3) mui = mk(d.muR[i * 9 + w * 3], d.muR[i * 9 + w * 3 + 1], d.muR[i * 9 + w * 3 + 2]);
     const R rc2 = sc<R>(p).rc2;
@@ -929,9 +993,9 @@ __global__ void __launch_bounds__(32 * NW, NW == 5 ? 3 : (NW == 3 ? (PER ? 5 : 6
 #pragma unroll
         for (int s = 0; s < NP; ++s) {
             if (!((bits >> s) & 1u)) continue;
-            if (s < 3) q.put((ta + pa++) % PQ_A, j, s, rs[s]);
-            else if (s < NS) q.put(PQ_A + (tm + pm++) % PQ_M, j, s, rs[s]);
-            else q.put(PQ_A + PQ_M + (tl + pl++) % PQ_L, j, s - NS, rs[s]);
+            if (s < 3) q.put((ta + pa++) % PQ_A, j * 8 + s, rs[s]);
+            else if (s < NS) q.put(PQ_A + (tm + pm++) % PQ_M, j * 8 + s, rs[s]);
+            else q.put(PQ_A + PQ_M + (tl + pl++) % PQ_L, j * 8 + s - NS, rs[s]);
         }
         ta += na;
         tm += nm;
@@ -969,9 +1033,8 @@ __global__ void __launch_bounds__(32 * NW, NW == 5 ? 3 : (NW == 3 ? (PER ? 5 : 6
     if (lane < 3) dst = d.gpt + (i * NP + w) * 3 + lane;
     else if (lane < 6) dst = d.gmu + (i * NS + w) * 3 + lane - 3;
     else if (lane < 12) dst = d.gth + (i * NS + w) * 6 + lane - 6;
-    if (dst) *dst += ke * double(s);
+    if (dst) *dst += (lane < 6 ? ke : ke * (1.0 / 3.0)) * double(s);
     if (VIR) {   // the warps' virials summed in a fixed order
-        __shared__ double s_w[NW][9];
         const R wv = warp_transpose_sum<R, 9>(A.W, reinterpret_cast<R *>(&q), lane);
         if (lane < 9) s_w[wq][lane] = double(wv);
         __syncthreads();
@@ -986,19 +1049,13 @@ __global__ void __launch_bounds__(32 * NW, NW == 5 ? 3 : (NW == 3 ? (PER ? 5 : 6
 template <typename R>
 void launch_real_polforce(const KParams &p, DevState<R> &d, Launch L) {
     if (p.vir) {
-        if (p.periodic) k_real_polforce<R, true, true, 0, NS><<<p.M, 32 * NS, 0, L.s>>>(p, d);
-        else k_real_polforce<R, false, true, 0, NS><<<p.M, 32 * NS, 0, L.s>>>(p, d);
-        count(L);
-        return;
-    }
-    if (p.periodic) {
-        k_real_polforce<R, true, false, 0, 3><<<p.M, 96, 0, L.s>>>(p, d);
-        k_real_polforce<R, true, false, 3, 2><<<p.M, 64, 0, L.s>>>(p, d);
+        if (p.periodic) k_real_polforce<R, true, true><<<p.M, 32 * NS, 0, L.s>>>(p, d);
+        else k_real_polforce<R, false, true><<<p.M, 32 * NS, 0, L.s>>>(p, d);
     } else {
-        k_real_polforce<R, false, false, 0, 3><<<p.M, 96, 0, L.s>>>(p, d);
-        k_real_polforce<R, false, false, 3, 2><<<p.M, 64, 0, L.s>>>(p, d);
+        if (p.periodic) k_real_polforce<R, true, false><<<p.M * NS, 32, 0, L.s>>>(p, d);
+        else k_real_polforce<R, false, false><<<p.M * NS, 32, 0, L.s>>>(p, d);
     }
-    count(L, 2);
+    count(L);
 }
 
 #define INST(R)                                                                                    \
