@@ -396,12 +396,24 @@ __device__ void item_du(const KParams &p, const Scal<R> &S, const ShortTables &T
 // VIR: also the virial, in the translation-invariance form of the pair
 // kernels (see vir_points_out): per item -1/2 (gradient on i's points) (x)
 // dO_ij, plus sum_p G_p (x) off_p at the end.
-// Resident blocks per SM: periodic 4 (repulsion) and 6 (dispersion), the
-// registers those need; gas phase 5 (measured faster for cluster batches).
-template <typename R, bool PER, int PART, bool VIR>
-__global__ void __launch_bounds__(128, PER ? (PART == 0 ? 4 : 6) : 5) k_short(KParams p, DevState<R> d) {
+// Resident blocks of four molecules per SM in FP32: periodic 4 (repulsion)
+// and 6 (dispersion), the registers those need; gas phase 5 (4096 clusters, both launches: 945 us,
+// 997 at 6).
+// FP64 is bound by the FP64 pipe, a quarter of it on each quarter of an SM,
+// so its warps are spread: one warp a block, and with fewer molecules than
+// quarters (SPLIT_MOL) SPL = 4 warps share a molecule's list (216 waters, both
+// launches: 907 us with four molecules a block, 772 with one, 486 shared;
+// 824 waters in clusters: 770, 592 and 632).
+template <typename R> constexpr int SW = sizeof(R) == 4 ? 4 : 1;   // molecules a block
+constexpr int SPL = 4, SPLIT_MOL = 608;
+
+template <typename R, bool PER, int PART, bool VIR, int NSP = 1>
+__global__ void __launch_bounds__(32 * SW<R> * NSP, sizeof(R) == 4 ? (PER ? (PART == 0 ? 4 : 6) : 5) : 8 / NSP)
+    k_short(KParams p, DevState<R> d) {
     __shared__ ShortTables T;
-    __shared__ int qbuf[4][SQ_WORDS];
+    __shared__ int qbuf[SW<R> * NSP][SQ_WORDS];
+    __shared__ double part[NSP > 1 ? NSP : 1][17];
+    static_assert(NSP == 1 || (SW<R> == 1 && !VIR), "a shared molecule has the block to itself");
     static_assert(SQ_D + SQ_CAPD <= SQ_WORDS && 15 * 33 * sizeof(R) <= SQ_WORDS * sizeof(int), "queue layout");
     static_assert(offsetof(KParams, xd_k) - offsetof(KParams, rep_k1) == offsetof(ShortTables, xd_k) &&
                       sizeof(ShortTables) == sizeof(KParams::Coef) * (9 * 4 + 27),
@@ -418,9 +430,9 @@ __global__ void __launch_bounds__(128, PER ? (PART == 0 ? 4 : 6) : 5) k_short(KP
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int *q = qbuf[w];
     const Scal<R> &S = sc<R>(p);
-    // molecules i = 4 block + w, then strided by the grid (a persistent launch
+    // molecules i = SW block + w, then strided by the grid (a persistent launch
     // with a capped grid leaves room for the kernels of the other streams)
-    for (int i = blockIdx.x * 4 + w; i < p.M; i += gridDim.x * 4) {
+    for (int i = NSP > 1 ? blockIdx.x : blockIdx.x * SW<R> + w; i < p.M; i += gridDim.x * SW<R>) {
         const R rc2 = S.rc2;
         ShortI<R> I;
         for (int k = 0; k < 3; ++k) I.P[k] = my_pt(d, i, k);
@@ -443,9 +455,9 @@ __global__ void __launch_bounds__(128, PER ? (PART == 0 ? 4 : 6) : 5) k_short(KP
         for (int k = 0; k < 9; ++k) acc.W[k] = R(0);
         int h[5] = {0, 0, 0, 0, 0}, t[5] = {0, 0, 0, 0, 0};   // heads and tails: BB, BL, LB, LL, D
         const int nn = d.nnbr[i];
-        for (int base = 0;; base += 32) {
+        for (int base = 0;; base += 32 * NSP) {
             const bool flush = base >= nn;
-            const int slot = base + lane;
+            const int slot = NSP > 1 ? base + lane * NSP + w : base + lane;
             const bool live = slot < nn;
             int j = 0;
             V3<R> dO = mk(R(0), R(0), R(0));
@@ -538,6 +550,22 @@ __global__ void __launch_bounds__(128, PER ? (PART == 0 ? 4 : 6) : 5) k_short(KP
                             acc.G[4].x, acc.G[4].y, acc.G[4].z};
         const R s = warp_transpose_sum<R, 15>(vals, reinterpret_cast<R *>(q), lane);
         const int pt = lane / 3;
+        if constexpr (NSP > 1) {   // the warps' sums in a fixed order
+            if (lane < 15) part[w][lane] = double(s);
+            const double e0 = warp_sum_acc(PART == 0 ? acc.Erep : acc.Ed), e1 = PART == 0 ? 0.0 : warp_sum_acc(acc.Ex);
+            if (lane == 0) part[w][15] = e0, part[w][16] = e1;
+            __syncthreads();
+            if (threadIdx.x < 17) {
+                double v = 0;
+                for (int k = 0; k < NSP; ++k) v += part[k][threadIdx.x];
+                const int q_ = threadIdx.x / 3;
+                if (threadIdx.x < 15) d.gpt[(i * NP + (q_ < 3 ? q_ : q_ + 2)) * 3 + threadIdx.x % 3] += v;
+                else if (threadIdx.x == 15) d.epart[i * NTERM + (PART == 0 ? T_REP : T_DISP)] += v;
+                else if (PART == 1) d.epart[i * NTERM + T_XDISP] += v;
+            }
+            __syncthreads();
+            continue;
+        }
         if (lane < 15) d.gpt[(i * NP + (pt < 3 ? pt : pt + 2)) * 3 + lane % 3] += double(s);
         if (VIR) vir_points_out(d, i, I.P, s, acc.W, reinterpret_cast<R *>(q), lane);
         if (PART == 0) {
@@ -559,7 +587,8 @@ __global__ void __launch_bounds__(128, PER ? (PART == 0 ? 4 : 6) : 5) k_short(KP
 // of the other streams.
 template <typename R>
 void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_blocks, int max_per_sm) {
-    unsigned nb = (p.M + 3) / 4;
+    constexpr int T = 32 * SW<R>;
+    unsigned nb = (p.M + SW<R> - 1) / SW<R>;
     if (max_blocks > 0 && nb > (unsigned)max_blocks) nb = (unsigned)max_blocks;
     size_t sm = 0;
     if (max_per_sm > 0 && !p.vir) {
@@ -582,18 +611,28 @@ void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_blocks, in
     count(L);
     if (p.vir) {
         if (p.periodic) {
-            k_short<R, true, 0, true><<<nb, 128, sm, L.s>>>(p, d);
-            k_short<R, true, 1, true><<<nb, 128, sm, L.s>>>(p, d);
+            k_short<R, true, 0, true><<<nb, T, sm, L.s>>>(p, d);
+            k_short<R, true, 1, true><<<nb, T, sm, L.s>>>(p, d);
         } else {
-            k_short<R, false, 0, true><<<nb, 128, sm, L.s>>>(p, d);
-            k_short<R, false, 1, true><<<nb, 128, sm, L.s>>>(p, d);
+            k_short<R, false, 0, true><<<nb, T, sm, L.s>>>(p, d);
+            k_short<R, false, 1, true><<<nb, T, sm, L.s>>>(p, d);
+        }
+    } else if (sizeof(R) == 8 && p.M < SPLIT_MOL) {
+        if constexpr (sizeof(R) == 8) {
+            if (p.periodic) {
+                k_short<R, true, 0, false, SPL><<<p.M, 32 * SPL, 0, L.s>>>(p, d);
+                k_short<R, true, 1, false, SPL><<<p.M, 32 * SPL, 0, L.s>>>(p, d);
+            } else {
+                k_short<R, false, 0, false, SPL><<<p.M, 32 * SPL, 0, L.s>>>(p, d);
+                k_short<R, false, 1, false, SPL><<<p.M, 32 * SPL, 0, L.s>>>(p, d);
+            }
         }
     } else if (p.periodic) {
-        k_short<R, true, 0, false><<<nb, 128, sm, L.s>>>(p, d);
-        k_short<R, true, 1, false><<<nb, 128, sm, L.s>>>(p, d);
+        k_short<R, true, 0, false><<<nb, T, sm, L.s>>>(p, d);
+        k_short<R, true, 1, false><<<nb, T, sm, L.s>>>(p, d);
     } else {
-        k_short<R, false, 0, false><<<nb, 128, sm, L.s>>>(p, d);
-        k_short<R, false, 1, false><<<nb, 128, sm, L.s>>>(p, d);
+        k_short<R, false, 0, false><<<nb, T, sm, L.s>>>(p, d);
+        k_short<R, false, 1, false><<<nb, T, sm, L.s>>>(p, d);
     }
     count(L, 2);
 }
