@@ -759,8 +759,7 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
     const KParams &p = ctx->kp;
     Launch L{ctx->s, &ctx->launches};
     Launch L2{ctx->s2, &ctx->launches};
-    launch_begin(d.scal, d.flags, tol, L);
-    { Phase ph(ctx, "sites");  launch_sites(p, d, L); }
+    { Phase ph(ctx, "sites");  launch_sites(p, d, tol, L); }
     const size_t ng = (size_t)p.K[0] * p.K[1] * p.K[2];
     sibfa_status st;
     if (p.periodic) {
@@ -811,7 +810,7 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
     if (!dipoles_only && !bg_short) { Phase ph(ctx, "short");  launch_short(p, d, L); }
     if (p.periodic) {
         if ((st = join_rec(ctx))) return st;
-        launch_merge_rec(p, d, L);
+        if (ctx->loop.ncta == 0) launch_merge_rec(p, d, L);   // the solve kernel merges itself
     }
     if (!dipoles_only) {
         if (!bg_ct) {
@@ -838,6 +837,18 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
     // the lambdas of the charge transfer feed k_pol_energy's working-precision copy
     if ((st = join_ct(ctx))) return st;
     launch_pol_energy(p, d, L);
+    // the energy totals, on the short-range kernels' stream behind them where
+    // those have one: beside the force pass
+    auto totals = [&](Launch Le) {
+        if (p.n_cl > 1) launch_cluster_energy(p, d, ctx->d_energy, Le);
+        else launch_energy_reduce(p.M, d.epart, d.epart_r, (sizeof(R) == 4 && p.periodic) ? d.eintra : nullptr,
+                                  d.epartial, d.counter + 1, ctx->d_energy, Le);
+    };
+    if (bg_short) {
+        if ((st = fork_short(ctx))) return st;
+        ctx->short_pending = true;
+        totals(Launch{ctx->s3, &ctx->launches});
+    }
     if (want_forces) {
         if (p.periodic) {
             // induced dipoles and charge-transfer lambdas in reciprocal space,
@@ -865,9 +876,7 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
         { Phase ph(ctx, "finalize");  launch_finalize(p, d, ctx->d_forces, L); }
     }
     if ((st = join_short(ctx))) return st;
-    if (p.n_cl > 1) launch_cluster_energy(p, d, ctx->d_energy, L);
-    else launch_energy_reduce(p.M, d.epart, d.epart_r, (sizeof(R) == 4 && p.periodic) ? d.eintra : nullptr,
-                              d.epartial, ctx->d_energy, L);
+    if (!bg_short) totals(L);
     return st_solve;
 }
 

@@ -333,27 +333,12 @@ __global__ void __launch_bounds__(PB) k_pcg_step(KParams p, DevState<R> d, cudaG
 
 static inline unsigned nblk(int n) { return (unsigned)((n + PB - 1) / PB); }
 
-// start of an evaluation: clear the solver scalars and the converged flag,
-// set the tolerance (error flags accumulate over the evaluations of one call)
-__global__ void k_begin(double *scal, int *flags, double tol_D) {
-    if (threadIdx.x < 16) scal[threadIdx.x] = 0.0;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        scal[S_TOL] = tol_D;
-        flags[1] = 0;   // PCG converged (integer copy of scal[S_DONE] for the loop kernels)
-    }
-}
 // after the solve: record a solve that stopped at the iteration limit
 __global__ void k_pcg_check(const double *scal, int *flags) {
     if (scal[S_DONE] == 0.0) atomicOr(flags, F_NOCONV);
 }
 void launch_pcg_check(const double *scal, int *flags, Launch L) {
     k_pcg_check<<<1, 1, 0, L.s>>>(scal, flags);
-    count(L);
-}
-
-void launch_begin(double *scal, int *flags, double tol_D, Launch L) {
-    k_begin<<<1, 32, 0, L.s>>>(scal, flags, tol_D);
     count(L);
 }
 
@@ -453,63 +438,111 @@ __device__ inline void frame_vjp(V3<W> zv, V3<W> xv, V3<W> gx, V3<W> gy, V3<W> g
     gzv = iz * (gz - dot(gz, ez) * ez);
 }
 
-// Four lanes per molecule.  Lane f < 3 carries the multipole sensitivities
+// Eight molecules a block.  All threads first sum the accumulators of the
+// streams in FP64 and bring them and the frames' inputs to shared memory in
+// the working precision, coalesced (the sums read by four diverging lanes a
+// molecule, as one dependent load after another, took 78 us at 32,000 waters and 21
+// at 8); then four lanes of the first warp take each molecule.
+// Lane f < 3 carries the multipole sensitivities
 // of the sites in frame f (frame 0: O and the lone pairs; frame 1: H1, M1;
 // frame 2: H2, M2) back through that frame's construction; lane 3 takes the
 // point gradients (lone-pair charge-transfer term, V_int chain rule,
 // midpoints, lone-pair carrier).  The four partial atom gradients are summed
-// with shuffles.  The accumulated gradients are summed in FP64 and the chain
-// rule runs in the working precision R, on the same frames as the site
-// kernel.
+// with shuffles.  The chain rule runs in the working precision R, on the same
+// frames as the site kernel.
+constexpr int FM = 8;   // molecules per block
+template <typename R>
+struct FinIn {
+    R G[FM][NP][3], mu[FM][NS][3], th[FM][NS][6], dv[FM][2][3];   // gradients, sensitivities, d V_lp
+    R ml[FM][NS * NMP], off[FM][NP][3], q[FM][NS], lam[FM][2], kap[FM][3];
+};
+// A thread's elements of one array of PER values a molecule (stride apart)
+template <int PER, typename T = double>
+struct FinLoad {
+    static constexpr int N = (FM * PER + 127) / 128;
+    T v[N];
+    __device__ __forceinline__ FinLoad(const T *a, int m0, int nm, int stride = 1) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const int e = k * 128 + threadIdx.x;
+            v[k] = e < nm * PER ? a[((size_t)m0 * PER + e) * stride] : T(0);
+        }
+    }
+    __device__ __forceinline__ void add(const FinLoad &o) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[k] += o.v[k];
+    }
+    template <typename R> __device__ __forceinline__ void put(R *out, int nm) const {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (k * 128 + (int)threadIdx.x < nm * PER) out[k * 128 + threadIdx.x] = R(v[k]);
+    }
+};
 template <typename R>
 __global__ void __launch_bounds__(128) k_finalize(KParams p, DevState<R> d, double *forces) {
-    const int gidx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int m = gidx >> 2, t = gidx & 3;
-    const bool live = m < p.M;
+    __shared__ FinIn<R> S;
+    const int m0 = blockIdx.x * FM, nm = min(FM, p.M - m0);
+    // every load first, so that they are all in flight together
+    FinLoad<NP * 3> g(d.gpt, m0, nm), gr(d.gpt_r, m0, nm), gs(d.gpt_s, m0, nm);
+    FinLoad<NS * 3> u(d.gmu, m0, nm), ur(d.gmu_r, m0, nm);
+    FinLoad<NS * 6> h(d.gth, m0, nm), hr(d.gth_r, m0, nm);
+    FinLoad<6> dv(d.dvlp, m0, nm), dvr(d.dvlp_r, m0, nm);
+    FinLoad<NS * NMP> ml(d.mp_local, m0, nm);
+    FinLoad<2> lam(d.lam, m0, nm);
+    FinLoad<3> kap(d.kap, m0, nm);
+    FinLoad<NP * 3, R> off(d.off, m0, nm);
+    FinLoad<NS, R> q(d.gmp, m0, nm, GMP);
+    g.add(gr);
+    g.add(gs);
+    u.add(ur);
+    h.add(hr);
+    dv.add(dvr);
+    g.put(&S.G[0][0][0], nm);
+    u.put(&S.mu[0][0][0], nm);
+    h.put(&S.th[0][0][0], nm);
+    dv.put(&S.dv[0][0][0], nm);
+    ml.put(&S.ml[0][0], nm);
+    lam.put(&S.lam[0][0], nm);
+    kap.put(&S.kap[0][0], nm);
+    off.put(&S.off[0][0][0], nm);
+    q.put(&S.q[0][0], nm);
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const int l = threadIdx.x >> 2, t = threadIdx.x & 3, m = m0 + l;
+    const bool live = l < nm;
     V3<R> gO = mk(R(0), R(0), R(0)), gH1 = gO, gH2 = gO;
     R W[9] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0)};   // virial (p.vir)
     if (live) {
         V3<R> r1, r2;
         bond_vectors(d.pos + m * 9, r1, r2);
         const R s1 = rsqrt_<R>(dot(r1, r1)), s2 = rsqrt_<R>(dot(r2, r2));
-        auto sum2 = [&](const double *a, const double *b, int o) {
-            return mk(R(a[o] + b[o]), R(a[o + 1] + b[o + 1]), R(a[o + 2] + b[o + 2]));
-        };
-        auto gpt = [&](int k) {
-            const int o = (m * NP + k) * 3;
-            return mk(R(d.gpt[o] + d.gpt_r[o] + d.gpt_s[o]), R(d.gpt[o + 1] + d.gpt_r[o + 1] + d.gpt_s[o + 1]),
-                      R(d.gpt[o + 2] + d.gpt_r[o + 2] + d.gpt_s[o + 2]));
-        };
+        auto vec = [](const R *a) { return mk(a[0], a[1], a[2]); };
+        auto gpt = [&](int k) { return vec(S.G[l][k]); };
         // lone-pair point gradient including the charge-transfer dependence through its potential
-        auto glp = [&](int l) {
-            return gpt(5 + l) + R(d.lam[m * 2 + l]) * sum2(d.dvlp, d.dvlp_r, (m * 2 + l) * 3);
-        };
+        auto glp = [&](int k) { return gpt(5 + k) + S.lam[l][k] * vec(S.dv[l][k]); };
         if (t < 3) {
             const int f = t;
             V3<R> zv, xv, E[3];
             frame_generators(f, r1, r2, s1, s2, zv, xv);
             frame_axes(zv, xv, E[0], E[1], E[2]);
             V3<R> gE[3] = {mk(R(0), R(0), R(0)), mk(R(0), R(0), R(0)), mk(R(0), R(0), R(0))};
-            for (int s = 0; s < NS; ++s) {
-                if (site_frame(s) != f) continue;
-                const double *ml = d.mp_local + (m * NS + s) * NMP;
-                const int ot = (m * NS + s) * 6;
-                const V3<R> gmu = sum2(d.gmu, d.gmu_r, (m * NS + s) * 3);
-                const double *gt6 = d.gth + ot, *gr6 = d.gth_r + ot;
-                const Sym<R> D{R(gt6[0] + gr6[0]), R(gt6[1] + gr6[1]), R(gt6[2] + gr6[2]),
-                               R(gt6[3] + gr6[3]), R(gt6[4] + gr6[4]), R(gt6[5] + gr6[5])};
-                const R tl[3][3] = {{R(ml[4]), R(ml[7]), R(ml[8])}, {R(ml[7]), R(ml[5]), R(ml[9])},
-                                    {R(ml[8]), R(ml[9]), R(ml[6])}};
+            for (int h = 0; h < (f == 0 ? 1 : 2); ++h) {   // the frame's sites: O; H1, M1; H2, M2
+                const int s = f + 2 * h;
+                const R *ml = S.ml[l] + s * NMP, *g6 = S.th[l][s];
+                const V3<R> gmu = vec(S.mu[l][s]);
+                const Sym<R> D{g6[0], g6[1], g6[2], g6[3], g6[4], g6[5]};
+                const R tl[3][3] = {{ml[4], ml[7], ml[8]}, {ml[7], ml[5], ml[9]}, {ml[8], ml[9], ml[6]}};
+#pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     const V3<R> acc = tl[k][0] * E[0] + tl[k][1] * E[1] + tl[k][2] * E[2];
-                    gE[k] = gE[k] + R(ml[1 + k]) * gmu + R(2) * symv(D, acc);
+                    gE[k] = gE[k] + ml[1 + k] * gmu + R(2) * symv(D, acc);
                 }
             }
             if (f == 0)   // lone pairs: X = O + d (-c z_O +/- s y_O)
-                for (int l = 0; l < 2; ++l) {
-                    const V3<R> G = glp(l);
+                for (int k = 0; k < 2; ++k) {
+                    const V3<R> G = glp(k);
                     gE[2] = gE[2] + R(-p.d_lp * p.lp_cos) * G;
-                    gE[1] = gE[1] + R(l == 0 ? p.d_lp * p.lp_sin : -p.d_lp * p.lp_sin) * G;
+                    gE[1] = gE[1] + R(k == 0 ? p.d_lp * p.lp_sin : -p.d_lp * p.lp_sin) * G;
                 }
             V3<R> gzv, gxv;
             frame_vjp(zv, xv, gE[0], gE[1], gE[2], gzv, gxv);
@@ -538,21 +571,22 @@ __global__ void __launch_bounds__(128) k_finalize(KParams p, DevState<R> d, doub
             }
         } else {
             V3<R> G[NS], X[NS];
+#pragma unroll
             for (int k = 0; k < NS; ++k) {
                 G[k] = gpt(k);
-                const R *o = d.off + (m * NP + k) * 3;
-                X[k] = mk(o[0], o[1], o[2]);
+                X[k] = vec(S.off[l][k]);
             }
             // charge-transfer dependence through the intramolecular potentials V_int(O, H1, H2)
+#pragma unroll
             for (int a = 0; a < 3; ++a) {
-                const double k = d.kap[m * 3 + a];
-                if (k == 0.0) continue;
-                const R kk = R(k * p.ke);
+                const R kk = S.kap[l][a] * R(p.ke);
+                if (kk == R(0)) continue;
+#pragma unroll
                 for (int s = 0; s < NS; ++s) {
                     if (s == a) continue;
                     const V3<R> dd = X[a] - X[s];
                     const R ir = rsqrt_<R>(dot(dd, dd));
-                    const R c = kk * d.gmp[(m * NS + s) * GMP] * ir * ir * ir;
+                    const R c = kk * S.q[l][s] * ir * ir * ir;
                     G[a] = G[a] - c * dd;
                     G[s] = G[s] + c * dd;
                     if (p.vir) vir_add(W, dd, dd, -c);   // the (a, s) pair's gradient on a is -c dd
@@ -562,10 +596,7 @@ __global__ void __launch_bounds__(128) k_finalize(KParams p, DevState<R> d, doub
             // the strain; they follow the frame of O instead, which lane 0's
             // chain rule has taken: remove their point share g_lp (x) off_lp.
             if (p.vir)
-                for (int l = 0; l < 2; ++l) {
-                    const R *o = d.off + (m * NP + 5 + l) * 3;
-                    vir_add(W, glp(l), mk(o[0], o[1], o[2]), R(-1));
-                }
+                for (int k = 0; k < 2; ++k) vir_add(W, glp(k), vec(S.off[l][5 + k]), R(-1));
             // midpoints and the lone pairs' carrier
             gO = G[0] + R(0.5) * (G[3] + G[4]) + glp(0) + glp(1);
             gH1 = G[1] + R(0.5) * G[3];
@@ -580,6 +611,7 @@ __global__ void __launch_bounds__(128) k_finalize(KParams p, DevState<R> d, doub
     }
     if (live && t == 0 && forces) {
         double *F = forces + m * 9;
+#pragma unroll
         for (int k = 0; k < 9; ++k) F[k] = -(double)v[k];
     }
     if (p.vir) {
@@ -651,20 +683,22 @@ void launch_merge_rec(const KParams &p, DevState<R> &d, Launch L) {
 
 template <typename R>
 void launch_finalize(const KParams &p, DevState<R> &d, double *forces_out, Launch L) {
-    const long long n = (long long)p.M * 4;
-    k_finalize<R><<<(unsigned)((n + 127) / 128), 128, 0, L.s>>>(p, d, forces_out);
+    k_finalize<R><<<(p.M + FM - 1) / FM, 128, 0, L.s>>>(p, d, forces_out);
     count(L);
 }
 
 // energy totals: out[k] = sum_m epart[m*NTERM + k], out[NTERM] = total, in a
-// fixed order: ER_BLOCKS blocks each sum a contiguous slice of molecules
+// fixed order: up to ER_BLOCKS blocks each sum a contiguous slice of molecules
 // (threads take independent chains, then a shared-memory tree per term) into
-// partials; one small block sums the partials in block order.
+// partials; the last block to finish sums the partials, one warp per term.
 constexpr int ER_BLOCKS = 128, ER_THREADS = 256;
-__global__ void __launch_bounds__(ER_THREADS) k_energy_partial(int M, const double *epart, const double *epart_r,
-                                                              const double *eintra, double *partial) {
+__global__ void __launch_bounds__(ER_THREADS) k_energy(int M, const double *epart, const double *epart_r,
+                                                      const double *eintra, double *partial, unsigned *counter,
+                                                      double *out) {
     __shared__ double sh[ER_THREADS / 32][NTERM];
-    const int per = (M + ER_BLOCKS - 1) / ER_BLOCKS;
+    __shared__ double tot[NTERM];
+    __shared__ bool last;
+    const int nb = gridDim.x, per = (M + nb - 1) / nb;
     const int m0 = blockIdx.x * per, m1 = min(M, m0 + per);
     double v[NTERM];
 #pragma unroll
@@ -677,9 +711,7 @@ __global__ void __launch_bounds__(ER_THREADS) k_energy_partial(int M, const doub
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
     for (int k = 0; k < NTERM; ++k) {
-        double x = v[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        const double x = warp_sum(v[k]);
         if (l == 0) sh[w][k] = x;
     }
     __syncthreads();
@@ -688,62 +720,73 @@ __global__ void __launch_bounds__(ER_THREADS) k_energy_partial(int M, const doub
         for (int j = 0; j < ER_THREADS / 32; ++j) x += sh[j][threadIdx.x];
         partial[blockIdx.x * NTERM + threadIdx.x] = x;
     }
-}
-__global__ void k_energy_final(const double *partial, double *out) {
-    __shared__ double sh[NTERM];
-    if (threadIdx.x < NTERM) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == (unsigned)nb - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    static_assert(NTERM <= ER_THREADS / 32, "one warp per term");
+    if (w < NTERM) {
         double x = 0.0;
-        for (int b = 0; b < ER_BLOCKS; ++b) x += partial[b * NTERM + threadIdx.x];
-        out[threadIdx.x] = x;
-        sh[threadIdx.x] = x;
+        for (int b = l; b < nb; b += 32) x += __ldcg(partial + b * NTERM + w);
+        x = warp_sum(x);
+        if (l == 0) {
+            out[w] = x;
+            tot[w] = x;
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int k = 0; k < NTERM; ++k) tot += sh[k];
-        out[NTERM] = tot;
+        double e = 0.0;
+        for (int k = 0; k < NTERM; ++k) e += tot[k];
+        out[NTERM] = e;
+        *counter = 0;
     }
 }
 
 void launch_energy_reduce(int M, const double *epart, const double *epart_r, const double *eintra, double *partial,
-                          double *out, Launch L) {
-    k_energy_partial<<<ER_BLOCKS, ER_THREADS, 0, L.s>>>(M, epart, epart_r, eintra, partial);
-    k_energy_final<<<1, 32, 0, L.s>>>(partial, out);
-    count(L, 2);
+                          unsigned *counter, double *out, Launch L) {
+    const int nb = std::max(1, std::min(ER_BLOCKS, M / ER_THREADS));
+    k_energy<<<nb, ER_THREADS, 0, L.s>>>(M, epart, epart_r, eintra, partial, counter, out);
+    count(L);
 }
 
 // Cluster batches: terms per cluster (one block per cluster, fixed order),
 // then their sums over the clusters into out (NTERM terms and the total).
 template <typename R>
-__global__ void k_cluster_energy(KParams p, DevState<R> d) {
-    __shared__ double sh[32];
-    const int c = blockIdx.x;
+__global__ void __launch_bounds__(128) k_cluster_energy(KParams p, DevState<R> d) {
+    const int c = blockIdx.x * 4 + (threadIdx.x >> 5), l = threadIdx.x & 31;   // one warp a cluster
+    if (c >= p.n_cl) return;
     const int m0 = d.cl_start[c], m1 = d.cl_start[c + 1];
+    double v[NTERM];
+#pragma unroll
+    for (int k = 0; k < NTERM; ++k) v[k] = 0.0;
+    for (int m = m0 + l; m < m1; m += 32)
+#pragma unroll
+        for (int k = 0; k < NTERM; ++k) v[k] += d.epart[m * NTERM + k] + d.epart_r[m * NTERM + k];
     double tot = 0;
+#pragma unroll
     for (int k = 0; k < NTERM; ++k) {
-        double v = 0;
-        for (int m = m0 + threadIdx.x; m < m1; m += blockDim.x) v += d.epart[m * NTERM + k] + d.epart_r[m * NTERM + k];
-        v = block_sum(v, sh);
-        if (threadIdx.x == 0) {
-            d.cl_energy[c * (NTERM + 1) + k] = v;
-            tot += v;
-        }
+        v[k] = warp_sum(v[k]);
+        tot += v[k];
+        if (l == 0) d.cl_energy[c * (NTERM + 1) + k] = v[k];
     }
-    if (threadIdx.x == 0) d.cl_energy[c * (NTERM + 1) + NTERM] = tot;
+    if (l == 0) d.cl_energy[c * (NTERM + 1) + NTERM] = tot;
 }
-__global__ void k_cluster_total(int n_cl, const double *cl_energy, double *out) {
+// one block per term (and the total)
+__global__ void __launch_bounds__(512) k_cluster_total(int n_cl, const double *cl_energy, double *out) {
     __shared__ double sh[32];
-    for (int k = 0; k <= NTERM; ++k) {
-        double v = 0;
-        for (int c = threadIdx.x; c < n_cl; c += blockDim.x) v += cl_energy[c * (NTERM + 1) + k];
-        v = block_sum(v, sh);
-        if (threadIdx.x == 0) out[k] = v;
-    }
+    const int k = blockIdx.x;
+    double v = 0;
+    for (int c = threadIdx.x; c < n_cl; c += blockDim.x) v += cl_energy[c * (NTERM + 1) + k];
+    v = block_sum(v, sh);
+    if (threadIdx.x == 0) out[k] = v;
 }
 template <typename R>
 void launch_cluster_energy(const KParams &p, DevState<R> &d, double *out, Launch L) {
-    k_cluster_energy<R><<<p.n_cl, 64, 0, L.s>>>(p, d);
-    k_cluster_total<<<1, 512, 0, L.s>>>(p.n_cl, d.cl_energy, out);
+    k_cluster_energy<R><<<(p.n_cl + 3) / 4, 128, 0, L.s>>>(p, d);
+    k_cluster_total<<<NTERM + 1, 512, 0, L.s>>>(p.n_cl, d.cl_energy, out);
     count(L, 2);
 }
 

@@ -14,11 +14,16 @@ namespace sibfa {
 // and rotation in the working precision R (the results are stored in R);
 // the SPME grid coordinates and the wrap in FP64.
 template <typename R>
-__global__ void __launch_bounds__(128) k_sites(KParams p, DevState<R> d) {
+__global__ void __launch_bounds__(128) k_sites(KParams p, DevState<R> d, double tol_D) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    // start of an evaluation: the solver's scalars (and the solve kernel's
+    // counter among them) and the converged flag
+    if (g < 16) d.scal[g] = g == SC_TOL ? tol_D : 0.0;
+    if (g == 0) d.flags[1] = 0;
     const int m = g >> 3, t = g & 7;
     const bool live = m < p.M;
     float ext = 0.f;
+    int move = 0;
     // bond vectors r1 = H1 - O, r2 = H2 - O: lane t < 6 takes one FP64
     // difference (rounded once to R) and the molecule's 8 lanes share them
     R bc = R(0);
@@ -129,6 +134,16 @@ __global__ void __launch_bounds__(128) k_sites(KParams p, DevState<R> d) {
                 }
                 d.ofw[m * 3 + k] = (float)v;
             }
+            // Verlet skin: squared O move since the last list build (the
+            // largest, as float bits: non-negative floats order like them)
+            if (p.periodic) {
+                double d2 = 0.0;
+                for (int k = 0; k < 3; ++k) {
+                    const double v = x[k] - d.oref[m * 3 + k];
+                    d2 += v * v;
+                }
+                move = __float_as_int((float)fmin(d2, 1e30));
+            }
         }
         // clear the per-molecule accumulators of this evaluation
         for (int k = t; k < NP * 3; k += 8)
@@ -148,16 +163,18 @@ __global__ void __launch_bounds__(128) k_sites(KParams p, DevState<R> d) {
         if (p.vir)
             for (int k = t; k < 9; k += 8) d.vir[m * 9 + k] = 0.0, d.vir_r[m * 9 + k] = 0.0;
     }
-    // largest point distance from its O (list margin): one atomic per warp
-    const int e = __reduce_max_sync(0xffffffffu, __float_as_int(ext));
-    if ((threadIdx.x & 31) == 0) atomicMax((int *)d.ext, e);
+    // largest point distance from its O (list margin) and O move: one atomic each per warp
+    const int e = __reduce_max_sync(0xffffffffu, __float_as_int(ext)), mv = __reduce_max_sync(0xffffffffu, move);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax((int *)d.ext, e);
+        if (p.periodic) atomicMax((int *)(d.lst + 2), mv);
+    }
 }
 
 template <typename R>
-void launch_sites(const KParams &p, DevState<R> &d, Launch L) {
-    cudaMemsetAsync(d.ext, 0, sizeof(float), L.s);
+void launch_sites(const KParams &p, DevState<R> &d, double tol_D, Launch L) {
     const long long n = (long long)p.M * 8;
-    k_sites<R><<<(unsigned)((n + 127) / 128), 128, 0, L.s>>>(p, d);
+    k_sites<R><<<(unsigned)((n + 127) / 128), 128, 0, L.s>>>(p, d, tol_D);
     count(L);
 }
 
@@ -170,28 +187,14 @@ void launch_sites(const KParams &p, DevState<R> &d, Launch L) {
 // kernels do no FP64 work.  Candidates are tested in FP32 with a small
 // margin; only accepted pairs pay the FP64 displacement.
 // ---------------------------------------------------------------------------
-__device__ inline double list_cut(const KParams &p, const float *ext) {
-    return p.periodic ? p.rc + 2.0 * (double)(*ext) : 1e300;
-}
 // the radius of a build: rc + 2 ext + the skin chosen at that build
 template <typename R>
 __device__ inline double build_cut(const KParams &p, const DevState<R> &d) {
     return p.periodic ? p.rc + 2.0 * (double)d.lst[0] + (double)d.lst[1] : 1e300;
 }
 
-// Verlet skin (periodic systems).  The largest O displacement since the last
-// build (squared, as float bits: non-negative floats order like their bits).
-template <typename R>
-__global__ void k_skin_disp(KParams p, DevState<R> d) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= p.M) return;
-    double d2 = 0.0;
-    for (int k = 0; k < 3; ++k) {
-        const double v = d.pos[m * 9 + k] - d.oref[m * 3 + k];
-        d2 += v * v;
-    }
-    atomicMax((int *)(d.lst + 2), __float_as_int((float)fmin(d2, 1e30)));
-}
+// Verlet skin (periodic systems), one thread.  Error flag for an extent that
+// the cutoff and box do not allow.
 // Rebuild when no list exists yet, when the skin is zero, or when twice the
 // largest move plus twice the growth of the site extent reaches the skin (a
 // pair can then have come from outside the listed radius to inside rc +
@@ -200,6 +203,11 @@ __global__ void k_skin_disp(KParams p, DevState<R> d) {
 template <typename R>
 __global__ void k_skin_decide(KParams p, DevState<R> d) {
     const float ext = *d.ext;
+    *d.ext = 0.f;   // for the next evaluation's maximum
+    if (p.periodic) {
+        const double half = 0.5 * fmin(p.box[0], fmin(p.box[1], p.box[2]));
+        if (p.rc + 2.0 * (double)ext > half || ext > 1.3f) atomicOr(d.flags, F_CUTOFF);
+    }
     const float md = sqrtf(__int_as_float(*(const int *)(d.lst + 2)));
     const bool rebuild = d.lflag[1] == 0 || d.lst[1] <= 0.f || 2.f * md + 2.f * fmaxf(0.f, ext - d.lst[0]) >= d.lst[1];
     if (rebuild) {
@@ -212,14 +220,6 @@ __global__ void k_skin_decide(KParams p, DevState<R> d) {
     *(int *)(d.lst + 2) = 0;
 }
 
-
-template <typename R>
-__global__ void k_check_ext(KParams p, DevState<R> d) {
-    if (!p.periodic) return;
-    double cut = list_cut(p, d.ext);
-    double half = 0.5 * fmin(p.box[0], fmin(p.box[1], p.box[2]));
-    if (cut > half || *d.ext > 1.3f) atomicOr(d.flags, F_CUTOFF);
-}
 
 // Minimum-image O_j - O_i from the fixed-point fractional coordinates (FP32).
 template <typename R>
@@ -266,21 +266,20 @@ __device__ inline void store_entry(const KParams &p, DevState<R> &d, int i, int 
 
 // Without a rebuild: the listed pairs' displacements at the current positions.
 template <typename R>
-__global__ void k_nbr_refresh(KParams p, DevState<R> d) {
-    if (d.lflag[0]) return;
-    const int i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    const int lane = threadIdx.x & 31;
-    if (i >= p.M) return;
+__device__ inline void refresh(const KParams &p, DevState<R> &d, int i, int lane) {
     const int nn = d.nnbr[i];
     for (int slot = lane; slot < nn; slot += 32) store_entry(p, d, i, slot, d.nbr[i * MAXN + slot]);
 }
 
 template <typename R>
 __global__ void k_nbr_all(KParams p, DevState<R> d) {
-    if (!d.lflag[0]) return;
     const int i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x & 31;
     if (i >= p.M) return;
+    if (!d.lflag[0]) {
+        refresh(p, d, i, lane);
+        return;
+    }
     if (lane < 3) d.oref[i * 3 + lane] = d.pos[i * 9 + lane];
     const double cut = build_cut(p, d) + 1e-3;
     const float cut2f = p.periodic ? (float)(cut * cut) : 3.0e38f;
@@ -406,10 +405,13 @@ __global__ void k_cell_sort(DevState<R> d, int ncell) {
 
 template <typename R>
 __global__ void k_nbr_cell(KParams p, DevState<R> d, int nc0, int nc1, int nc2) {
-    if (!d.lflag[0]) return;
     const int i = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x & 31;
     if (i >= p.M) return;
+    if (!d.lflag[0]) {
+        refresh(p, d, i, lane);
+        return;
+    }
     if (lane < 3) d.oref[i * 3 + lane] = d.pos[i * 9 + lane];
     const double cut = build_cut(p, d) + 1e-3;
     const float cut2f = (float)(cut * cut);
@@ -441,14 +443,10 @@ __global__ void k_nbr_cell(KParams p, DevState<R> d, int nc0, int nc1, int nc2) 
 
 template <typename R>
 void launch_neighbors(const KParams &p, DevState<R> &d, int nc[3], Launch L) {
-    k_check_ext<R><<<1, 1, 0, L.s>>>(p, d);
-    k_skin_disp<R><<<(p.M + 255) / 256, 256, 0, L.s>>>(p, d);
     k_skin_decide<R><<<1, 1, 0, L.s>>>(p, d);
-    count(L, 3);
-    const int wpb = 4;
-    // either the refresh or the build kernels do work, as the decision says
-    k_nbr_refresh<R><<<(p.M + wpb - 1) / wpb, 32 * wpb, 0, L.s>>>(p, d);
     count(L);
+    const int wpb = 4;
+    // the list kernel builds or refreshes, as the decision says
     if (!p.periodic || nc[0] < 3 || nc[1] < 3 || nc[2] < 3) {
         k_nbr_all<R><<<(p.M + wpb - 1) / wpb, 32 * wpb, 0, L.s>>>(p, d);
         count(L);
@@ -464,8 +462,8 @@ void launch_neighbors(const KParams &p, DevState<R> &d, int nc[3], Launch L) {
     count(L, 5);
 }
 
-template void launch_sites<float>(const KParams &, DevState<float> &, Launch);
-template void launch_sites<double>(const KParams &, DevState<double> &, Launch);
+template void launch_sites<float>(const KParams &, DevState<float> &, double, Launch);
+template void launch_sites<double>(const KParams &, DevState<double> &, double, Launch);
 template void launch_neighbors<float>(const KParams &, DevState<float> &, int *, Launch);
 template void launch_neighbors<double>(const KParams &, DevState<double> &, int *, Launch);
 

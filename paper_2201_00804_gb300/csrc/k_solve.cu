@@ -639,6 +639,7 @@ __global__ void __launch_bounds__(LT, sizeof(R) == 4 ? 2 : 1)
 #pragma unroll 1
     for (int e = tid; e < n9; e += LT) {
         const int k = m0 * 9 + e;
+        if (PER) d.efield[k] += d.efield_r[k];   // the reciprocal chain's part
         double m;
         if (guess.n > 0) {
             m = 0;

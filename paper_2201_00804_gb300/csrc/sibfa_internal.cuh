@@ -815,7 +815,8 @@ struct Launch {
     uint64_t *count;
 };
 
-template <typename R> void launch_sites(const KParams &p, DevState<R> &d, Launch L);
+// sites and frames; also starts the evaluation (accumulators, solver scalars, tolerance)
+template <typename R> void launch_sites(const KParams &p, DevState<R> &d, double tol_D, Launch L);
 template <typename R> void launch_neighbors(const KParams &p, DevState<R> &d, int ncell[3], Launch L);
 template <typename R> void launch_real_perm(const KParams &p, DevState<R> &d, Launch L);
 template <typename R> void launch_lp_potential(const KParams &p, DevState<R> &d, Launch L);
@@ -874,7 +875,7 @@ template <typename R> void launch_pcg_step(const KParams &p, DevState<R> &d, Lau
                                            cudaGraphConditionalHandle loop = 0, int maxit = 0);
 template <typename R> void launch_pol_energy(const KParams &p, DevState<R> &d, Launch L);
 void launch_energy_reduce(int M, const double *epart, const double *epart_r, const double *eintra, double *partial,
-                          double *out, Launch L);
+                          unsigned *counter, double *out, Launch L);
 // mixed periodic path: the intramolecular Ewald energy of every molecule in FP64 into eintra
 template <typename R> void launch_intra_energy64(const KParams &p, DevState<R> &d, Launch L);
 // k-space virial sums of one convolution pass (0: permanent, 1: force pass) fused with the convolution
@@ -882,7 +883,6 @@ template <typename R> void launch_convolve_vir(const KParams &p, DevState<R> &d,
 // out[9] = -dE/d eps summed over molecules, both chains and the k-space partials
 template <typename R> void launch_virial_total(const KParams &p, DevState<R> &d, double *out, Launch L);
 template <typename R> void launch_cluster_energy(const KParams &p, DevState<R> &d, double *out, Launch L);
-void launch_begin(double *scal, int *flags, double tol_D, Launch L);
 void launch_pcg_check(const double *scal, int *flags, Launch L);
 void launch_water_intra(int M, const double *pos, double *F, double kb, double r0, double ka, double th0, int anh,
                         double kub, double rub, Launch L);
