@@ -89,8 +89,8 @@ typedef struct {
      * pointer, n_clusters+1 ints, cluster_start[0] = 0, cluster_start
      * [n_clusters] = n_mol, increasing; copied at create).  Molecules of
      * different clusters do not interact; each call evaluates every cluster
-     * with one launch per kernel, the polarization solve stops when the RMS
-     * residual of every cluster is below pcg_tol_D, sibfa_cluster_terms
+     * with one launch per kernel, the polarization solve ends with the RMS
+     * residual of every cluster below pcg_tol_D, sibfa_cluster_terms
      * returns the terms per cluster and the terms of sibfa_energy_forces are
      * their sums.  n_clusters = 0 or 1: one system (cluster_start unused). */
     int n_clusters;
@@ -182,8 +182,9 @@ typedef struct sibfa_ctx sibfa_ctx;
  * influence function and FFT plans, allocates all device state.  *out is
  * NULL on failure.  The PCG loop runs on the device: for one system of up to
  * some 1700 waters, on a grid whose axes are products of 2, 3 and 5, as one
- * cooperative kernel, otherwise as a CUDA graph with a conditional
- * while-node.  With the environment variable SIBFA_PCG_HOST_LOOP=1 at
+ * cooperative kernel, for gas-phase clusters of up to 64 waters on the mixed
+ * path as one block per cluster (each cluster stops on its own residual),
+ * otherwise as a CUDA graph with a conditional while-node.  With the environment variable SIBFA_PCG_HOST_LOOP=1 at
  * creation it is driven from the host instead (one launch per kernel and
  * iteration), which kernel profilers can follow.  The context tunes the schedule of its short-range kernels
  * (resident blocks per SM, and whether they finish before the polarization

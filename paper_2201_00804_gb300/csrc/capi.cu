@@ -66,6 +66,7 @@ struct sibfa_ctx {
     uint64_t pcg_iter_launches = 0;
     uint64_t pcg_graph_solves = 0;   // graph solves whose iteration count is not yet folded into launches
     LoopPlan loop;               // solve in one kernel (ncta > 0)
+    int cluster_max = 0;         // > 0: every cluster solves on its own (largest cluster a batch may hold)
     bool capturing = false;
     int prec = SIBFA_PREC_MIXED;
     DevState<float> df{};
@@ -349,6 +350,7 @@ void fill_params(KParams &k, const sibfa_params &P, const sibfa_run_opts &o, int
     k.rc = o.rc;
     k.rc2 = o.rc * o.rc;
     k.skin = o.periodic ? LIST_SKIN : 0.0;
+    k.tlist = 1;
     k.ct_orig = o.ct_original ? 1 : 0;
     k.alpha = o.ewald_alpha;
     for (int i = 0; i < 3; ++i) k.K[i] = o.grid[i];
@@ -677,6 +679,17 @@ sibfa_status solve(sibfa_ctx *ctx, DevState<R> &d, double tol, Launch L, bool fu
     const KParams &p = ctx->kp;
     const int warm = (ctx->opts.warm_start && ctx->have_mu) ? 1 : 0;
     const MuGuess g = mu_guess(ctx, full);
+    if constexpr (sizeof(R) == 4) {
+        if (ctx->cluster_max > 0) {
+            double *push = mu_slot(ctx, full);
+            CK(launch_pcg_cluster(p, d, ctx->cluster_max, ctx->opts.pcg_max_iter > 0 ? ctx->opts.pcg_max_iter : 200, g,
+                                  warm, push, L));
+            if (push) mu_pushed(ctx);
+            CK(cudaMemcpyAsync(ctx->h_scal, d.scal, 16 * sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
+            ctx->have_mu = true;
+            return SIBFA_OK;
+        }
+    }
     if (ctx->loop.ncta > 0) {
         // serial profiling: the real-space product alone (its result is not used)
         if (ctx->serial) {
@@ -1069,7 +1082,7 @@ sibfa_status create_impl(sibfa_ctx *ctx, const sibfa_topology *topo) {
     // the solve in one kernel: one system whose grid axes factor into small
     // primes (cluster batches stop on each cluster's residual; the host loop
     // is for profilers)
-    if (ctx->kp.n_cl == 1 && ctx->pcg_graph_state != -1) {
+    if (ctx->kp.n_cl == 1 && ctx->pcg_graph_state != -1 && ctx->cluster_max == 0) {
         int dev = 0, n_sm = 0;
         CK(cudaGetDevice(&dev));
         CK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
@@ -1304,10 +1317,16 @@ sibfa_status sibfa_create(const sibfa_params *params, const sibfa_topology *topo
             nmax = std::min(MAXN, std::max(1, big - 1));
         }
         ctx->kp.tls = 3 * nmax;
-    }
-    {
+        // small gas-phase clusters of the mixed path: one block each, which
+        // recomputes the products and needs no pair list
         const char *e = getenv("SIBFA_PCG_HOST_LOOP");
         if (e && e[0] == '1') ctx->pcg_graph_state = -1;
+        else if (!opts->periodic && opts->precision == SIBFA_PREC_MIXED && nmax + 1 <= CLUSTER_MAX) {
+            ctx->cluster_max = nmax + 1;
+            ctx->kp.tlist = 0;
+        }
+    }
+    {
         const char *t = getenv("SIBFA_TUNE");
         if (t && t[0] == '0') ctx->tune.on = false;
     }

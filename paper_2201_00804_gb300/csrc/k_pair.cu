@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(VIR ? 32 * NS : 32,
         if (!PER) os = my_pt(d, j, s);
         R g1 = R(0), T2 = R(0);
         perm_pair<R, PER, AT, VIR>(p, T, ms, s, q.at(e), os, acc, g1, T2, x);
-        if (AT && w < 3) {
+        if (AT && w < 3 && p.tlist) {
             // the same atom pair in the polarization matrix T: the field of a
             // dipole mu at x is T2 (mu.x) x + g1 mu = sgn(T2) (mu.y) y + g1 mu
             // with y = sqrt|T2| x: four values and the sign in the index's top bit

@@ -843,6 +843,173 @@ __global__ void __launch_bounds__(LT, sizeof(R) == 4 ? 2 : 1)
     if (tid == 0 && s_lost) atomicOr(d.flags, F_TIMEOUT);
 }
 
+// ---------------------------------------------------------------------------
+// Gas phase, FP32 products: one block solves one cluster on its own, with the
+// usual conjugate gradients and its own step lengths; it stops when its
+// residual is below the tolerance.  The product recomputes the Thole kernels
+// from the molecules' displacements in shared memory (about 45 instructions a
+// pair) instead of streaming the pair list: on 4096 clusters of 2-32 waters a
+// product streamed 260 MB in 81 us, ten of them a solve, and every iteration
+// waited for the slowest cluster twice (1430 us a solve).  The vectors stay in
+// FP64; their arithmetic is about as long as the products here, on the FP64 pipe
+// beside them.
+// ---------------------------------------------------------------------------
+constexpr int CT = 128;   // threads
+
+// sums of one value per thread, left in out[0..NV): fewer FP64 instructions
+// than shuffles in every warp
+template <int NV>
+__device__ inline void block_totals(const double (&v)[NV], double (*sh)[CT], double *out, int tid) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) sh[k][tid] = v[k];
+    __syncthreads();
+    const int w = tid >> 5, l = tid & 31;
+    if (w < NV) {
+        const double x = warp_sum((sh[w][l] + sh[w][l + 32]) + (sh[w][l + 64] + sh[w][l + 96]));
+        if (l == 0) out[w] = x;
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(CT, 8)
+    k_pcg_cluster(KParams p, DevState<float> d, int maxit, MuGuess guess, int warm, double *push) {
+    __shared__ double sh[2][CT];
+    __shared__ double s_sum[2], s_val[2];
+    const int tid = threadIdx.x;
+    const int m0 = d.cl_start[blockIdx.x], n = d.cl_start[blockIdx.x + 1] - m0, n3 = n * 3, n9 = n * 9;
+    double *mu = reinterpret_cast<double *>(loop_raw), *r = mu + n9, *pv = r + n9, *ap = pv + n9;
+    float4 *u = reinterpret_cast<float4 *>(loop_raw + ((4 * n9 * sizeof(double) + 15) & ~(size_t)15));
+    float *off = reinterpret_cast<float *>(u + n3), *ef = off + n9, *D = ef + n9;
+    // lanes per row: the largest power of two that fits the block
+    int P = 1;
+    while (2 * P * n3 <= CT && P < 16) P *= 2;
+    const int part = tid & (P - 1);
+    // offsets of the atoms, and O_j - O_i of every (i, j != i) in the list's order
+    for (int e = tid; e < n9; e += CT) off[e] = d.off[(size_t)(m0 + e / 9) * NP * 3 + e % 9];
+    for (int e = tid; e < n * (n - 1) * 3; e += CT) {
+        const int i = e / ((n - 1) * 3), k = e - i * (n - 1) * 3;
+        D[e] = d.ndo[(size_t)(m0 + i) * MAXN * 3 + k];
+    }
+    for (int e = tid; e < n9; e += CT) {
+        const int k = m0 * 9 + e;
+        double m;
+        if (guess.n > 0) {
+            m = 0;
+            for (int j = 0; j < guess.n; ++j) m += guess.c[j] * guess.h[j][k];
+        } else {
+            m = warm ? d.mu[k] : p.a_pol[(e / 3) % 3] * d.efield[k];
+        }
+        mu[e] = m;
+        reinterpret_cast<float *>(u)[e / 3 * 4 + e % 3] = float(m);
+    }
+    // field of the dipoles u of the other molecules at every atom
+    auto field = [&]() {
+        __syncthreads();
+        for (int r0 = 0; r0 < n3; r0 += CT / P) {
+            const int row = r0 + tid / P;
+            float ex = 0.f, ey = 0.f, ez = 0.f;
+            if (row < n3) {
+                const int i = row / 3, a = row - i * 3;
+                const float ox = off[row * 3], oy = off[row * 3 + 1], oz = off[row * 3 + 2];
+                const float k0 = p.sf.thole * p.ainv3f[a][0], k1 = p.sf.thole * p.ainv3f[a][1];
+                for (int jj = part; jj < n - 1; jj += P) {
+                    const int j = jj + (jj >= i);
+                    const float *dd = D + (i * (n - 1) + jj) * 3;
+                    const float dx = dd[0], dy = dd[1], dz = dd[2];
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) {
+                        const float *os = off + (j * 3 + b) * 3;
+                        const float4 m = u[j * 3 + b];
+                        const float x = (ox - os[0]) - dx, y = (oy - os[1]) - dy, z = (oz - os[2]) - dz;
+                        const float r2 = x * x + y * y + z * z, ri = rsqrt_(r2), r2i = ri * ri;
+                        const float b1 = ri * r2i, t = (b == 0 ? k0 : k1) * r2 * (r2 * ri), e = exp_(-t);
+                        const float T1 = b1 - e * b1, b2 = 3.f * b1 * r2i, T2 = b2 - (e + t * e) * b2;
+                        const float c = T2 * (m.x * x + m.y * y + m.z * z);
+                        ex += c * x - T1 * m.x;
+                        ey += c * y - T1 * m.y;
+                        ez += c * z - T1 * m.z;
+                    }
+                }
+            }
+            for (int o = P >> 1; o > 0; o >>= 1) {
+                ex += __shfl_xor_sync(0xffffffffu, ex, o);
+                ey += __shfl_xor_sync(0xffffffffu, ey, o);
+                ez += __shfl_xor_sync(0xffffffffu, ez, o);
+            }
+            if (row < n3 && part == 0) ef[row * 3] = ex, ef[row * 3 + 1] = ey, ef[row * 3 + 2] = ez;
+        }
+        __syncthreads();
+    };
+    const double tol = d.scal[SC_TOL] / 4.80321, tol2 = tol * tol * n3;   // bound of the sum of squares
+    field();
+    double v2[2] = {0, 0};
+    for (int e = tid; e < n9; e += CT) {
+        const int c = (e / 3) % 3;
+        const double al = p.a_pol[c], q = d.efield[m0 * 9 + e] - (mu[e] * p.a_pol_inv[c] - double(ef[e])), z = al * q;
+        r[e] = q;
+        pv[e] = z;
+        reinterpret_cast<float *>(u)[e / 3 * 4 + e % 3] = float(z);
+        v2[0] += q * z;
+        v2[1] += z * z;
+    }
+    block_totals<2>(v2, sh, s_sum, tid);
+    double rz = s_sum[0];
+    int it = 0;
+    bool done = s_sum[1] < tol2;
+    while (!done && it < maxit) {
+        field();
+        double v1[1] = {0};
+        for (int e = tid; e < n9; e += CT) {
+            const double pe = pv[e], q = pe * p.a_pol_inv[(e / 3) % 3] - double(ef[e]);
+            ap[e] = q;
+            v1[0] += pe * q;
+        }
+        block_totals<1>(v1, sh, s_sum, tid);
+        if (tid == 0) s_val[0] = rz / s_sum[0];
+        __syncthreads();
+        const double a = s_val[0];
+        v2[0] = v2[1] = 0;
+        for (int e = tid; e < n9; e += CT) {
+            mu[e] += a * pv[e];
+            const double q = r[e] - a * ap[e], z = p.a_pol[(e / 3) % 3] * q;
+            r[e] = q;
+            v2[0] += q * z;
+            v2[1] += z * z;
+        }
+        block_totals<2>(v2, sh, s_sum, tid);
+        if (tid == 0) s_val[1] = s_sum[0] / rz;
+        __syncthreads();
+        const double beta = s_val[1];
+        rz = s_sum[0];
+        ++it;
+        done = s_sum[1] < tol2;
+        for (int e = tid; e < n9; e += CT) {
+            const double q = p.a_pol[(e / 3) % 3] * r[e] + beta * pv[e];
+            pv[e] = q;
+            reinterpret_cast<float *>(u)[e / 3 * 4 + e % 3] = float(q);
+        }
+    }
+    // The last residual is at hand: one more Jacobi step costs no product and
+    // leaves the dipoles closer (the batch used to iterate until its slowest
+    // cluster was done, which over-converged the others).
+    for (int e = tid; e < n9; e += CT) {
+        const double m = mu[e] + p.a_pol[(e / 3) % 3] * r[e];
+        d.mu[m0 * 9 + e] = m;
+        if (push) push[m0 * 9 + e] = m;
+    }
+    if (tid == 0) {   // the batch reports its largest iteration count and residual (non-negative doubles order like their bits)
+        atomicMax((unsigned long long *)(d.scal + SC_IT), (unsigned long long)__double_as_longlong((double)it));
+        atomicMax((unsigned long long *)(d.scal + SC_RES),
+                  (unsigned long long)__double_as_longlong(sqrt(s_sum[1] / n3) * 4.80321));
+        if (!done) atomicOr(d.flags, F_NOCONV);
+    }
+}
+
+size_t cluster_smem(int n) {
+    return (((size_t)n * 9 * 4 * sizeof(double) + 15) & ~(size_t)15) + (size_t)n * 3 * sizeof(float4) +
+           ((size_t)n * 18 + (size_t)n * (n - 1) * 3) * sizeof(float);
+}
+
 // Passes of an axis of n points; false when a prime above 5 is left.  FP64
 // takes radix 2 for every factor of 2: a pass costs its longest thread's FP64
 // instructions times some 73 cycles (a warp-wide one on its quarter of the SM),
@@ -942,6 +1109,18 @@ cudaError_t launch_pcg_loop(const KParams &p, DevState<R> &d, const LoopPlan &lp
     count(L);
     return p.periodic ? cudaLaunchKernelEx(&cfg, k_pcg_loop<R, true>, p, d, lp, g, warm, push)
                       : cudaLaunchKernelEx(&cfg, k_pcg_loop<R, false>, p, d, lp, g, warm, push);
+}
+
+cudaError_t launch_pcg_cluster(const KParams &p, DevState<float> &d, int nmax, int maxit, const MuGuess &g, int warm,
+                               double *push, Launch L) {
+    const size_t sm = cluster_smem(nmax);
+    if (sm > 40000) {
+        const cudaError_t e = cudaFuncSetAttribute(k_pcg_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+    }
+    k_pcg_cluster<<<p.n_cl, CT, sm, L.s>>>(p, d, maxit, g, warm, push);
+    count(L);
+    return cudaGetLastError();
 }
 
 #define INST(R)                                                                                              \

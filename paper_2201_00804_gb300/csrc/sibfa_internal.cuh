@@ -51,6 +51,7 @@ struct KParams {
     int n_cl;              // clusters (1: one system)
     int tls;               // T-pair list slots per polarizable atom: 3 x the most neighbours a molecule can have
     int vir;               // 1: this evaluation also accumulates the virial
+    int tlist;             // 1: the permanent pass records the polarization pair list
     int ct_orig;           // 1: the original many-body charge transfer (acceptor potentials kept)
     double box[3];
     double ibox[3];        // 1 / box

@@ -65,6 +65,24 @@ def test_one_kernel_matches_the_separate_kernels(kind, size, grid, fp64, monkeyp
     assert f <= (1e-8 if fp64 else 1e-5), f
 
 
+@pytest.mark.parametrize("sizes", [[1], [1, 2, 3, 42, 43, 64], [2] * 40 + [5, 8, 11, 21, 22, 32], [64, 64, 1]])
+def test_clusters_on_their_own_match_the_batch_solve(sizes, monkeypatch):
+    """Mixed path: each cluster's own solve (lanes per row from 16 down to 1,
+    clusters up to the largest it takes) against the batch-wide one."""
+    import paper_2201_00804_gb300 as pkg
+    s, start, _ = synth.make_cluster_sizes(sizes, seed=31)
+    kw = dict(periodic=False) if len(sizes) == 1 else dict(periodic=False, cluster_start=start)
+    tol = 1e-7
+    a = _mu(pkg, s, kw, tol, pkg.PREC_MIXED)
+    monkeypatch.setenv("SIBFA_PCG_HOST_LOOP", "1")
+    b = _mu(pkg, s, kw, tol, pkg.PREC_MIXED)
+    for c in range(len(sizes)):
+        x, y = (v[0][start[c] * 9:start[c + 1] * 9] for v in (a, b))
+        assert float(np.sqrt(((x - y) ** 2).sum() / (x.size / 3))) * 4.80321 <= 8 * tol + MIXED_MU_RMS_D, c
+    assert a[2] < tol
+    assert np.linalg.norm(a[4] - b[4]) <= 1e-5 * max(np.linalg.norm(b[4]), 1e-30)
+
+
 def test_iteration_limit_is_reported():
     import paper_2201_00804_gb300 as pkg
     s, o = synth.make_config("water216")
