@@ -66,7 +66,19 @@ struct sibfa_ctx {
     uint64_t pcg_iter_launches = 0;
     uint64_t pcg_graph_solves = 0;   // graph solves whose iteration count is not yet folded into launches
     LoopPlan loop;               // solve in one kernel (ncta > 0)
+    LoopPlan conv;               // grid convolution in one kernel (ncta > 0)
     int cluster_max = 0;         // > 0: every cluster solves on its own (largest cluster a batch may hold)
+    // whole evaluations as CUDA graphs (small systems): one per kind of call
+    struct EvalGraph {
+        bool forces, dipoles, warm;
+        int vir, cap, join;
+        double tol;
+        int seen = 0;                // evaluations of this kind
+        cudaGraphExec_t exec = nullptr;
+        uint64_t launches = 0;       // kernels of one replay
+    };
+    std::vector<EvalGraph> eval_graphs;
+    bool eval_graph_off = false;     // a capture failed: launch by launch from then on
     bool capturing = false;
     int prec = SIBFA_PREC_MIXED;
     DevState<float> df{};
@@ -228,6 +240,7 @@ sibfa_status alloc_state(sibfa_ctx *ctx, DevState<R> &d) {
     AL(d.epw, M * NS * 2);
     AL(d.vir, M * 9);
     AL(d.vir_r, M * 9);
+    AL(d.vir_s, M * 9);
     AL(d.vphi, M * 9);
     AL(d.gpt_r, M * NP * 3);
     AL(d.gpt_s, M * NP * 3);
@@ -568,6 +581,24 @@ sibfa_status fft(sibfa_ctx *ctx, DevState<R> &d, bool forward, int ngrid) {
     return SIBFA_OK;
 }
 
+// The grids' convolution with the influence function on s2 (permanent and
+// force passes): in one kernel for the small systems whose solve runs in one
+// too, where the chain of transforms is on the critical path (216 waters: 66 ->
+// 53 and 71 -> 58 us a pass, FP64 198 -> 162 and 247 -> 216); the library's
+// transforms otherwise (32,000 waters, products included: 8454 us a call
+// against 8597).
+template <typename R>
+sibfa_status convolve(sibfa_ctx *ctx, DevState<R> &d, int ngrid, Launch L2) {
+    if (ctx->conv.ncta > 0) {
+        CK(launch_grid_conv(ctx->kp, d, ctx->conv, ngrid, L2));
+        return SIBFA_OK;
+    }
+    sibfa_status st = fft(ctx, d, true, ngrid);
+    if (st) return st;
+    launch_convolve(ctx->kp, d, d.cgrid, ngrid, 0, L2);
+    return fft(ctx, d, false, ngrid);
+}
+
 // T vec (field part): real space into d.efp on s, reciprocal and
 // intramolecular into d.efp_r on s2, concurrently; vec is the PCG vector
 // already copied to d.vecR.
@@ -742,6 +773,73 @@ sibfa_status solve(sibfa_ctx *ctx, DevState<R> &d, double tol, Launch L, bool fu
 template <typename R>
 sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, double tol);
 
+void drop_eval_graphs(sibfa_ctx *ctx) {
+    for (auto &g : ctx->eval_graphs)
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+    ctx->eval_graphs.clear();
+}
+
+// An evaluation of a small system is some 30 short kernels on four streams,
+// and launching them one by one takes the host as long as they run (8 waters:
+// 132 us a call against some 80 on the device).  From the third evaluation of a kind
+// on (calls with the same outputs, tolerance, start and schedule) it is replayed
+// as a graph.  Only for solves in one kernel from the direct field or the
+// previous dipoles: a start from the dipole history names other buffers every
+// time.  The graph holds the context's own buffers and parameters only; a new
+// box or batch drops it.
+constexpr size_t EVAL_GRAPHS = 8;   // kinds kept at most
+constexpr int EVAL_GRAPH_MOL = 2000;   // above it the launches hide behind the kernels
+template <typename R>
+sibfa_status evaluate_graph(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, double tol, bool &ran) {
+    ran = false;
+    const bool one_kernel = ctx->loop.ncta > 0 || ctx->cluster_max > 0;
+    if (!one_kernel || ctx->eval_graph_off || ctx->profiling || ctx->opts.warm_start >= 2 || ctx->M > EVAL_GRAPH_MOL)
+        return SIBFA_OK;
+    if (!dipoles_only && !ctx->kp.vir && ctx->tune.on && ctx->tune.choice < 0) return SIBFA_OK;
+    const ShortSched sc = short_sched(ctx);
+    const bool warm = ctx->opts.warm_start && ctx->have_mu;
+    sibfa_ctx::EvalGraph *g = nullptr;
+    for (auto &e : ctx->eval_graphs)
+        if (e.forces == want_forces && e.dipoles == dipoles_only && e.warm == warm && e.vir == ctx->kp.vir &&
+            e.cap == sc.cap && e.join == (int)sc.join_before_solve && e.tol == tol)
+            g = &e;
+    if (!g) {
+        if (ctx->eval_graphs.size() >= EVAL_GRAPHS) drop_eval_graphs(ctx);
+        ctx->eval_graphs.push_back({want_forces, dipoles_only, warm, ctx->kp.vir, sc.cap, (int)sc.join_before_solve, tol});
+        g = &ctx->eval_graphs.back();
+    }
+    if (!g->exec) {
+        if (++g->seen < 3) return SIBFA_OK;
+        cudaGraph_t graph = nullptr;
+        const uint64_t before = ctx->launches;
+        if (cudaStreamBeginCapture(ctx->s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->eval_graph_off = true;
+            return SIBFA_OK;
+        }
+        ctx->capturing = true;
+        const sibfa_status a = evaluate_impl<R>(ctx, want_forces, dipoles_only, tol);
+        const sibfa_status b = join_short(ctx), c = join_ct(ctx);
+        ctx->capturing = false;
+        const cudaError_t e = cudaStreamEndCapture(ctx->s, &graph);
+        g->launches = ctx->launches - before;
+        ctx->launches = before;
+        if (a || b || c || e != cudaSuccess ||
+            cudaGraphInstantiate(&g->exec, graph, cudaGraphInstantiateFlagUseNodePriority) != cudaSuccess) {
+            g->exec = nullptr;
+            ctx->eval_graph_off = true;
+        }
+        if (graph) cudaGraphDestroy(graph);
+        cudaGetLastError();
+        if (!g->exec) return SIBFA_OK;
+    }
+    CK(cudaGraphLaunch(g->exec, ctx->s));
+    ctx->launches += g->launches;
+    ctx->have_mu = true;
+    ran = true;
+    return SIBFA_OK;
+}
+
 // One evaluation; the short-range stream is joined back on every path.
 // Full evaluations (not the dipole-only solve nor the virial variant) feed
 // the short-range autotuner.
@@ -754,6 +852,11 @@ sibfa_status evaluate(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, doubl
     if (timed) {
         tune_account(ctx);
         if (T.choice < 0) CK(cudaEventRecord(T.e0, ctx->s));
+    }
+    if (!timed || T.choice >= 0) {
+        bool ran = false;
+        const sibfa_status sg = evaluate_graph<R>(ctx, want_forces, dipoles_only, tol, ran);
+        if (sg || ran) return sg;
     }
     const sibfa_status st = evaluate_impl<R>(ctx, want_forces, dipoles_only, tol);
     const sibfa_status sj = join_short(ctx);
@@ -783,10 +886,13 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
         // the second grid takes the solve kernel's spreads
         CK(cudaMemsetAsync(d.grid, 0, (ctx->loop.ncta ? 2 : 1) * ng * sizeof(R), ctx->s2));
         launch_spread(p, d, SPREAD_PERM, nullptr, d.grid, L2);
-        if ((st = fft(ctx, d, true, 1))) return st;
-        if (p.vir) launch_convolve_vir(p, d, 0, L2);
-        else launch_convolve(p, d, d.cgrid, 1, 0, L2);
-        if ((st = fft(ctx, d, false, 1))) return st;
+        if (p.vir) {
+            if ((st = fft(ctx, d, true, 1))) return st;
+            launch_convolve_vir(p, d, 0, L2);
+            if ((st = fft(ctx, d, false, 1))) return st;
+        } else if ((st = convolve(ctx, d, 1, L2))) {
+            return st;
+        }
         launch_gather_perm(p, dr, L2);
         launch_intra_perm(p, dr, L2);
         if (ctx->serial && (st = join_rec(ctx))) return st;
@@ -795,9 +901,9 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
     // Short-range terms on the third, lowest-priority stream beside the
     // permanent pass and the solve (which is latency-bound and leaves SMs
     // idle): their short blocks fill in behind the other streams' work.  They
-    // write their own gradient array and are joined before the chain rule.
-    // The virial variant runs in order on the main stream.
-    const bool bg_short = !dipoles_only && !p.vir && !ctx->serial;
+    // write their own gradient (and virial) arrays and are joined before the
+    // chain rule.
+    const bool bg_short = !dipoles_only && !ctx->serial;
     if (bg_short) {
         if ((st = fork_short(ctx))) return st;
         ctx->short_pending = true;
@@ -813,14 +919,18 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
     // Lone-pair potentials and then the charge transfer on the fourth stream
     // (the transfer after the reciprocal chain); joined before the
     // polarization energy, which copies the lambdas.
-    const bool bg_ct = !dipoles_only && !p.vir && !ctx->serial;
+    const bool bg_ct = !dipoles_only && !ctx->serial;
     if (bg_ct) {
         if ((st = fork_ct(ctx))) return st;
         ctx->ct_pending = true;
         launch_lp_potential(p, d, Launch{ctx->s4, &ctx->launches});
     }
     { Phase ph(ctx, "real_perm");  launch_real_perm(p, d, L); }
-    if (!dipoles_only && !bg_short) { Phase ph(ctx, "short");  launch_short(p, d, L); }
+    if (!dipoles_only && !bg_short) {
+        Phase ph(ctx, "short");
+        DevState<R> ds = short_view(d);
+        launch_short(p, ds, L);
+    }
     if (p.periodic) {
         if ((st = join_rec(ctx))) return st;
         if (ctx->loop.ncta == 0) launch_merge_rec(p, d, L);   // the solve kernel merges itself
@@ -872,10 +982,13 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
             CK(cudaMemsetAsync(d.grid, 0, 2 * ng * sizeof(R), ctx->s2));
             launch_spread(p, d, SPREAD_DIP, nullptr, d.grid, L2);
             launch_spread(p, d, SPREAD_LAMBDA, nullptr, d.grid + ng, L2);
-            if ((sf = fft(ctx, d, true, 2))) return sf;
-            if (p.vir) launch_convolve_vir(p, d, 1, L2);
-            else launch_convolve(p, d, d.cgrid, 2, 0, L2);
-            if ((sf = fft(ctx, d, false, 2))) return sf;
+            if (p.vir) {
+                if ((sf = fft(ctx, d, true, 2))) return sf;
+                launch_convolve_vir(p, d, 1, L2);
+                if ((sf = fft(ctx, d, false, 2))) return sf;
+            } else if ((sf = convolve(ctx, d, 2, L2))) {
+                return sf;
+            }
             launch_gather_polforce(p, dr, L2);
             launch_intra_polforce(p, dr, L2);
             if (ctx->serial && (sf = join_rec(ctx))) return sf;
@@ -959,6 +1072,7 @@ sibfa_status set_box(sibfa_ctx *ctx, DevState<R> &d, const double *box) {
     launch_influence(k, d.infl, L);
     launch_influence_copy(k, d, L);
     CK(cudaMemsetAsync(d.lflag + 1, 0, sizeof(int), ctx->s));   // no list yet: rebuild
+    drop_eval_graphs(ctx);
     if (ctx->pcg_graph_state == 1) {
         cudaGraphExecDestroy(ctx->pcg_exec);
         ctx->pcg_exec = nullptr;
@@ -1094,17 +1208,21 @@ sibfa_status create_impl(sibfa_ctx *ctx, const sibfa_topology *topo) {
             AL(vec, (size_t)M * 12);
             lp.vec = vec;
             lp.maxit = ctx->opts.pcg_max_iter > 0 ? ctx->opts.pcg_max_iter : 200;
-            if (ctx->opts.periodic) {
-                const std::vector<double> t = loop_twiddles(ctx->kp.K);
-                const std::vector<R> tr(t.begin(), t.end());
-                R *tw = nullptr;
-                AL(tw, tr.size());
-                CK(cudaMemcpyAsync(tw, tr.data(), tr.size() * sizeof(R), cudaMemcpyHostToDevice, ctx->s));
-                CK(cudaStreamSynchronize(ctx->s));   // the host table is freed on return
-                lp.tw = tw;
-            }
             ctx->loop = lp;
         }
+    }
+    if (ctx->opts.periodic && ctx->loop.ncta > 0) {
+        const std::vector<double> t = loop_twiddles(ctx->kp.K);
+        const std::vector<R> tr(t.begin(), t.end());
+        R *tw = nullptr;
+        AL(tw, tr.size());
+        CK(cudaMemcpyAsync(tw, tr.data(), tr.size() * sizeof(R), cudaMemcpyHostToDevice, ctx->s));
+        CK(cudaStreamSynchronize(ctx->s));   // the host table is freed on return
+        int dev = 0, n_sm = 0;
+        CK(cudaGetDevice(&dev));
+        CK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+        conv_plan<R>(ctx->conv, ctx->kp.K, n_sm);
+        ctx->conv.tw = ctx->loop.tw = tw;
     }
     if (ctx->opts.periodic) {
         Launch L{ctx->s, &ctx->launches};
@@ -1547,6 +1665,7 @@ void sibfa_destroy(sibfa_ctx *ctx) {
     if (ctx->s2) cudaStreamSynchronize(ctx->s2);
     if (ctx->s3) cudaStreamSynchronize(ctx->s3);
     if (ctx->s4) cudaStreamSynchronize(ctx->s4);
+    drop_eval_graphs(ctx);
     if (ctx->pcg_exec) cudaGraphExecDestroy(ctx->pcg_exec);
     if (ctx->ev_fork4) cudaEventDestroy(ctx->ev_fork4);
     if (ctx->tune.e0) cudaEventDestroy(ctx->tune.e0);
@@ -1624,6 +1743,7 @@ sibfa_status ctx_set_batch(sibfa_ctx *ctx, int M, int n_cl, const int *cluster_s
     ctx->pcg_exec = nullptr;
     ctx->pcg_graph_state = -1;
     ctx->loop.ncta = 0;   // laid out for the first size
+    drop_eval_graphs(ctx);
     return SIBFA_OK;
 }
 

@@ -625,15 +625,15 @@ __global__ void __launch_bounds__(128) k_finalize(KParams p, DevState<R> d, doub
     }
 }
 
-// Virial total: out[3a + b] = -dE/d eps_ab = -(sum over molecules of both
-// chains' dE/d eps + the k-space sums of npass convolution passes), summed
+// Virial total: out[3a + b] = -dE/d eps_ab = -(sum over molecules of the
+// streams' dE/d eps + the k-space sums of npass convolution passes), summed
 // in a fixed order by one block.
 template <typename R>
 __global__ void __launch_bounds__(256) k_virial_total(int M, DevState<R> d, int npass, double *out) {
     __shared__ double sh[8][9];
     double v[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int m = threadIdx.x; m < M; m += blockDim.x)
-        for (int k = 0; k < 9; ++k) v[k] += d.vir[m * 9 + k] + d.vir_r[m * 9 + k];
+        for (int k = 0; k < 9; ++k) v[k] += d.vir[m * 9 + k] + d.vir_r[m * 9 + k] + d.vir_s[m * 9 + k];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int k = 0; k < 9; ++k) {
         double x = v[k];

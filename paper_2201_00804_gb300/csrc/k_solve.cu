@@ -21,6 +21,8 @@
 //   p = u + beta p, s = w + beta s, mu += a p, r -= a s,
 // the same iterates as the usual form; rz and the residual norm travel with
 // the barrier after the spread and u.w with the one after the gather.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 
@@ -115,12 +117,12 @@ __device__ inline int quo(int t, unsigned m) { return (int)__umulhi((unsigned)t,
 
 // One radix-r pass (self-sorting, decimation in frequency) over `lines`
 // transforms held as [index][line] with `ld` elements per index.
-template <int r, typename R, typename C>
+template <int NT, int r, typename R, typename C>
 __device__ inline void fft_pass(const C *in, C *out, const FftPass P, int lines, int ld, unsigned div_lines,
                                 const C *tw, unsigned sg, int tid) {
     const int sp = P.sp, m = P.m, tasks = lines * sp * m;
 #pragma unroll 1
-    for (int t = tid; t < tasks; t += LREC) {
+    for (int t = tid; t < tasks; t += NT) {
         const int i = quo(t, div_lines), l = t - i * lines;
         const int q0 = sp > 1 ? quo(i, P.div_sp) : i, q = i - q0 * sp;
         const C *v = in + i * ld + l;   // q + sp q0 = i
@@ -144,8 +146,9 @@ __device__ inline void fft_pass(const C *in, C *out, const FftPass P, int lines,
     }
 }
 
-// Named barrier of the reciprocal threads of a block
-__device__ inline void part_sync() { asm volatile("bar.sync 1, %0;" ::"n"(LREC) : "memory"); }
+// Named barrier of the NT threads that transform
+template <int NT>
+__device__ inline void part_sync() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
 
 // dynamic shared memory of the kernel
 extern __shared__ __align__(16) unsigned char loop_raw[];
@@ -153,7 +156,7 @@ extern __shared__ __align__(16) unsigned char loop_raw[];
 // All passes of one axis on the transform buffers at byte offsets ba and bb of
 // the block's shared memory (offsets, so that the accesses stay shared-space
 // ones); the data starts in ba, and the offset that holds the result is returned.
-template <typename R>
+template <int NT, typename R>
 __device__ __noinline__ int fft_lines(int ba, int bb, const FftAxis &A, int lines, int ld, unsigned div_lines, int tw_at,
                                       unsigned sg, int tid) {
     using C = typename Cplx<R>::T;
@@ -163,12 +166,12 @@ __device__ __noinline__ int fft_lines(int ba, int bb, const FftAxis &A, int line
         const FftPass &P = A.pass[k];
         const C *a = reinterpret_cast<const C *>(loop_raw + ba);
         C *b = reinterpret_cast<C *>(loop_raw + bb);
-        if (P.r == 8) fft_pass<8, R>(a, b, P, lines, ld, div_lines, tw, sg, tid);
-        else if (P.r == 4) fft_pass<4, R>(a, b, P, lines, ld, div_lines, tw, sg, tid);
-        else if (P.r == 5) fft_pass<5, R>(a, b, P, lines, ld, div_lines, tw, sg, tid);
-        else if (P.r == 3) fft_pass<3, R>(a, b, P, lines, ld, div_lines, tw, sg, tid);
-        else fft_pass<2, R>(a, b, P, lines, ld, div_lines, tw, sg, tid);
-        part_sync();
+        if (P.r == 8) fft_pass<NT, 8, R>(a, b, P, lines, ld, div_lines, tw, sg, tid);
+        else if (P.r == 4) fft_pass<NT, 4, R>(a, b, P, lines, ld, div_lines, tw, sg, tid);
+        else if (P.r == 5) fft_pass<NT, 5, R>(a, b, P, lines, ld, div_lines, tw, sg, tid);
+        else if (P.r == 3) fft_pass<NT, 3, R>(a, b, P, lines, ld, div_lines, tw, sg, tid);
+        else fft_pass<NT, 2, R>(a, b, P, lines, ld, div_lines, tw, sg, tid);
+        part_sync<NT>();
         const int t = ba;
         ba = bb;
         bb = t;
@@ -186,6 +189,20 @@ struct GridView {
     C *spec;
     const R *infl;
 };
+template <typename R>
+__device__ inline GridView<R> grid_view(const KParams &p, const DevState<R> &d, R *gs, R *gp, int buf, int tw, int nbuf) {
+    GridView<R> G;
+    G.K0 = p.K[0], G.K1 = p.K[1], G.K2 = p.K[2], G.nz = p.K[2] / 2 + 1;
+    G.L = (G.K1 + 1) / 2, G.ldz = G.L | 1;
+    G.b0 = buf;
+    G.b1 = buf + nbuf * (int)sizeof(typename Cplx<R>::T);
+    G.tw = tw;
+    G.gs = gs;
+    G.gp = gp;
+    G.spec = reinterpret_cast<typename Cplx<R>::T *>(d.cgrid);
+    G.infl = d.inflR;
+    return G;
+}
 constexpr int GL = 4;   // global loads a thread keeps in flight
 template <typename C>
 __device__ inline C *at(int off) { return reinterpret_cast<C *>(loop_raw + off); }
@@ -193,80 +210,81 @@ __device__ inline C *at(int off) { return reinterpret_cast<C *>(loop_raw + off);
 // n complex values, rows of `row` of them `pitch` apart in global memory, into
 // the buffer at b0, GL of a thread's loads in flight (an L2 access takes some
 // 0.4 us); columns past `live` are zero.
-template <typename R>
+template <int NT, typename R>
 __device__ inline void load_rows(const typename Cplx<R>::T *g, int n, int row, unsigned div_row, size_t pitch, int live,
                                  int b0, int tid) {
     using C = typename Cplx<R>::T;
     C *b = at<C>(b0);
-    for (int t0 = tid; t0 < n; t0 += GL * LREC) {
+    for (int t0 = tid; t0 < n; t0 += GL * NT) {
         C v[GL];
 #pragma unroll
         for (int u = 0; u < GL; ++u) {
-            const int t = t0 + u * LREC, x = quo(t, div_row), c = t - x * row;
+            const int t = t0 + u * NT, x = quo(t, div_row), c = t - x * row;
             v[u] = t < n && c < live ? g[x * pitch + c] : C{R(0), R(0)};
         }
 #pragma unroll
         for (int u = 0; u < GL; ++u)
-            if (t0 + u * LREC < n) b[t0 + u * LREC] = v[u];
+            if (t0 + u * NT < n) b[t0 + u * NT] = v[u];
     }
 }
 
 // Forward z and y transforms of plane x: two real lines along z go as the
-// real and imaginary part of one complex transform.  The plane is cleared for
-// the next spread.
-template <typename R>
+// real and imaginary part of one complex transform.  CLEAR: the plane is
+// cleared for the next spread.
+template <int NT, bool CLEAR, typename R>
 __device__ void plane_forward(const GridView<R> &G, const LoopPlan &lp, const FftAxis *ax, int x, int tid) {
     using C = typename Cplx<R>::T;
     const int n = G.L * G.K2, K2 = G.K2;
     R *g = G.gs + (size_t)x * G.K1 * K2;
     C *w = at<C>(G.b0);
-    for (int t0 = tid; t0 < n; t0 += GL * LREC) {
+    for (int t0 = tid; t0 < n; t0 += GL * NT) {
         C v[GL];
 #pragma unroll
         for (int u = 0; u < GL; ++u) {
-            const int t = t0 + u * LREC, l = quo(t, lp.div_k2);
+            const int t = t0 + u * NT, l = quo(t, lp.div_k2);
             const R *a = g + t + l * K2;   // line 2 l, point z = t - l K2
             v[u].x = t < n ? a[0] : R(0);
             v[u].y = t < n && 2 * l + 1 < G.K1 ? a[K2] : R(0);
         }
 #pragma unroll
         for (int u = 0; u < GL; ++u) {
-            const int t = t0 + u * LREC, l = quo(t, lp.div_k2);
+            const int t = t0 + u * NT, l = quo(t, lp.div_k2);
             if (t < n) w[(t - l * K2) * G.ldz + l] = v[u];
         }
     }
-    part_sync();
-    for (int t = tid; t < G.K1 * K2; t += LREC) g[t] = R(0);
-    const int ra = fft_lines<R>(G.b0, G.b1, ax[2], G.L, G.ldz, lp.div_l, G.tw, 0u, tid);
+    part_sync<NT>();
+    if (CLEAR)
+        for (int t = tid; t < G.K1 * K2; t += NT) g[t] = R(0);
+    const int ra = fft_lines<NT, R>(G.b0, G.b1, ax[2], G.L, G.ldz, lp.div_l, G.tw, 0u, tid);
     const int rb = ra == G.b0 ? G.b1 : G.b0;
     const C *a = at<C>(ra);
     C *b = at<C>(rb);
-    for (int t = tid; t < G.L * G.nz; t += LREC) {
+    for (int t = tid; t < G.L * G.nz; t += NT) {
         const int k = quo(t, lp.div_l), l = t - k * G.L;
         const C u = a[k * G.ldz + l], v = a[(k ? K2 - k : 0) * G.ldz + l];
         b[2 * l * G.nz + k] = {R(0.5) * (u.x + v.x), R(0.5) * (u.y - v.y)};
         if (2 * l + 1 < G.K1) b[(2 * l + 1) * G.nz + k] = {R(0.5) * (u.y + v.y), R(0.5) * (v.x - u.x)};
     }
-    part_sync();
-    b = at<C>(fft_lines<R>(rb, ra, ax[1], G.nz, G.nz, lp.div_nz, G.tw, 0u, tid));
+    part_sync<NT>();
+    b = at<C>(fft_lines<NT, R>(rb, ra, ax[1], G.nz, G.nz, lp.div_nz, G.tw, 0u, tid));
     const int m = G.K1 * G.nz;
     C *out = G.spec + (size_t)x * m;
-    for (int t = tid; t < m; t += LREC) out[t] = b[t];
-    part_sync();
+    for (int t = tid; t < m; t += NT) out[t] = b[t];
+    part_sync<NT>();
 }
 
 // The way back, into the potential grid.
-template <typename R>
+template <int NT, typename R>
 __device__ void plane_inverse(const GridView<R> &G, const LoopPlan &lp, const FftAxis *ax, int x, int tid) {
     using C = typename Cplx<R>::T;
     const int m = G.K1 * G.nz, n = G.L * G.K2;
-    load_rows<R>(G.spec + (size_t)x * m, m, G.nz, lp.div_nz, G.nz, G.nz, G.b0, tid);
-    part_sync();
-    const int ra = fft_lines<R>(G.b0, G.b1, ax[1], G.nz, G.nz, lp.div_nz, G.tw, 0x80000000u, tid);
+    load_rows<NT, R>(G.spec + (size_t)x * m, m, G.nz, lp.div_nz, G.nz, G.nz, G.b0, tid);
+    part_sync<NT>();
+    const int ra = fft_lines<NT, R>(G.b0, G.b1, ax[1], G.nz, G.nz, lp.div_nz, G.tw, 0x80000000u, tid);
     const int rb = ra == G.b0 ? G.b1 : G.b0;
     const C *a = at<C>(ra);
     C *b = at<C>(rb);
-    for (int t = tid; t < n; t += LREC) {
+    for (int t = tid; t < n; t += NT) {
         const int z = quo(t, lp.div_l), l = t - z * G.L;
         const bool up = z < G.nz;
         const int k = up ? z : G.K2 - z;
@@ -276,41 +294,41 @@ __device__ void plane_inverse(const GridView<R> &G, const LoopPlan &lp, const Ff
         if (!up) u.y = -u.y, v.y = -v.y;
         b[z * G.ldz + l] = {u.x - v.y, u.y + v.x};
     }
-    part_sync();
-    b = at<C>(fft_lines<R>(rb, ra, ax[2], G.L, G.ldz, lp.div_l, G.tw, 0x80000000u, tid));
+    part_sync<NT>();
+    b = at<C>(fft_lines<NT, R>(rb, ra, ax[2], G.L, G.ldz, lp.div_l, G.tw, 0x80000000u, tid));
     R *g = G.gp + (size_t)x * G.K1 * G.K2;
-    for (int t = tid; t < n; t += LREC) {
+    for (int t = tid; t < n; t += NT) {
         const int l = quo(t, lp.div_k2);
         const C v = b[(t - l * G.K2) * G.ldz + l];
         R *o = g + t + l * G.K2;
         o[0] = v.x;
         if (2 * l + 1 < G.K1) o[G.K2] = v.y;
     }
-    part_sync();
+    part_sync<NT>();
 }
 
 // x transforms of a tile of columns, the convolution, and back.
-template <typename R>
+template <int NT, typename R>
 __device__ void columns(const GridView<R> &G, const LoopPlan &lp, const FftAxis *ax, int tile, int tid) {
     using C = typename Cplx<R>::T;
     const int n = G.K1 * G.nz, xt = lp.xt, c0 = tile * xt, live = min(xt, n - c0), all = G.K0 * xt;
-    load_rows<R>(G.spec + c0, all, xt, lp.div_xt, n, live, G.b0, tid);
-    part_sync();
-    const int ra = fft_lines<R>(G.b0, G.b1, ax[0], xt, xt, lp.div_xt, G.tw, 0u, tid);
+    load_rows<NT, R>(G.spec + c0, all, xt, lp.div_xt, n, live, G.b0, tid);
+    part_sync<NT>();
+    const int ra = fft_lines<NT, R>(G.b0, G.b1, ax[0], xt, xt, lp.div_xt, G.tw, 0u, tid);
     C *a = at<C>(ra);
-    for (int t = tid; t < all; t += LREC) {
+    for (int t = tid; t < all; t += NT) {
         const int x = quo(t, lp.div_xt), c = t - x * xt;
         const R f = c < live ? G.infl[(size_t)x * n + c0 + c] : R(0);
         a[t].x *= f;
         a[t].y *= f;
     }
-    part_sync();
-    a = at<C>(fft_lines<R>(ra, ra == G.b0 ? G.b1 : G.b0, ax[0], xt, xt, lp.div_xt, G.tw, 0x80000000u, tid));
-    for (int t = tid; t < all; t += LREC) {
+    part_sync<NT>();
+    a = at<C>(fft_lines<NT, R>(ra, ra == G.b0 ? G.b1 : G.b0, ax[0], xt, xt, lp.div_xt, G.tw, 0x80000000u, tid));
+    for (int t = tid; t < all; t += NT) {
         const int x = quo(t, lp.div_xt), c = t - x * xt;
         if (c < live) G.spec[(size_t)x * n + c0 + c] = a[t];
     }
-    part_sync();
+    part_sync<NT>();
 }
 
 // Weights of an atom: x and y axis value (5) and derivative (5) at the grid
@@ -574,25 +592,17 @@ __global__ void __launch_bounds__(LT, sizeof(R) == 4 ? 2 : 1)
         __syncthreads();
     };
     auto chain = [&]() {
-        part_sync();
+        part_sync<LREC>();
         target += ncta;
         if (tid == 0 && !counter_wait(bar, target)) s_lost = 1;
-        part_sync();
+        part_sync<LREC>();
     };
 
 #pragma unroll 1
     for (int t = tid; t < nm * 3; t += LT) cnt[t] = d.tl_n[m0 * 3 + t];
     GridView<R> G{};
     if constexpr (PER) {
-        G.K0 = p.K[0], G.K1 = p.K[1], G.K2 = p.K[2], G.nz = p.K[2] / 2 + 1;
-        G.L = (G.K1 + 1) / 2, G.ldz = G.L | 1;
-        G.b0 = (int)mem.buf;
-        G.b1 = G.b0 + lp.nbuf * (int)sizeof(C);
-        G.tw = (int)mem.tw;
-        G.gp = d.grid;
-        G.gs = d.grid + (size_t)G.K0 * G.K1 * G.K2;
-        G.spec = reinterpret_cast<C *>(d.cgrid);
-        G.infl = d.inflR;
+        G = grid_view(p, d, d.grid + (size_t)p.K[0] * p.K[1] * p.K[2], d.grid, (int)mem.buf, (int)mem.tw, lp.nbuf);
         C *tw = reinterpret_cast<C *>(raw + mem.tw);
 #pragma unroll 1
         for (int t = tid; t < lp.ntw; t += LT) tw[t] = reinterpret_cast<const C *>(lp.tw)[t];
@@ -697,13 +707,13 @@ __global__ void __launch_bounds__(LT, sizeof(R) == 4 ? 2 : 1)
         }
         // T u: real space and, beside it, the reciprocal chain
         if (PER && tid < LREC) {
-            for (int x = blockIdx.x; x < G.K0; x += ncta) plane_forward(G, lp, s_ax, x, tid);
+            for (int x = blockIdx.x; x < G.K0; x += ncta) plane_forward<LREC, true>(G, lp, s_ax, x, tid);
             chain();
             if (!s_lost)
-                for (int t = blockIdx.x; t * lp.xt < G.K1 * G.nz; t += ncta) columns(G, lp, s_ax, t, tid);
+                for (int t = blockIdx.x; t * lp.xt < G.K1 * G.nz; t += ncta) columns<LREC>(G, lp, s_ax, t, tid);
             chain();
             if (!s_lost)
-                for (int x = blockIdx.x; x < G.K0; x += ncta) plane_inverse(G, lp, s_ax, x, tid);
+                for (int x = blockIdx.x; x < G.K0; x += ncta) plane_inverse<LREC>(G, lp, s_ax, x, tid);
             chain();
             // gather: lanes 0-4 of an atom's group the x-lines of its stencil,
             // lane 5 the self term, lanes 6 and 7 the other two atoms' erf field
@@ -841,6 +851,48 @@ __global__ void __launch_bounds__(LT, sizeof(R) == 4 ? 2 : 1)
         if (!done) atomicOr(d.flags, F_NOCONV);
     }
     if (tid == 0 && s_lost) atomicOr(d.flags, F_TIMEOUT);
+}
+
+// ---------------------------------------------------------------------------
+// Convolution of ngrid real grids (d.grid) with the influence function in one
+// cooperative kernel: the plane and column phases of the solve with all of a
+// block's threads.  As library transforms it is seven launches of 4 to 5 us
+// each at these sizes (55 us in FP64 at 24^3).
+// ---------------------------------------------------------------------------
+template <typename R>
+__global__ void __launch_bounds__(LT, sizeof(R) == 4 ? 2 : 1)
+    k_grid_conv(KParams p, DevState<R> d, LoopPlan lp, int ngrid) {
+    using C = typename Cplx<R>::T;
+    namespace cg = cooperative_groups;
+    cg::grid_group grid = cg::this_grid();
+    __shared__ FftAxis s_ax[3];
+    const int tid = threadIdx.x;
+    C *tw = reinterpret_cast<C *>(loop_raw);
+    for (int t = tid; t < lp.ntw; t += LT) tw[t] = reinterpret_cast<const C *>(lp.tw)[t];
+    if (tid < 3) s_ax[tid] = lp.ax[tid];
+    __syncthreads();
+    const size_t ng = (size_t)p.K[0] * p.K[1] * p.K[2];
+    GridView<R> G = grid_view(p, d, d.grid, d.grid, (int)((lp.ntw * sizeof(C) + 15) & ~(size_t)15), 0, lp.nbuf);
+    const int n = G.K1 * G.nz, tiles = (n + lp.xt - 1) / lp.xt;
+    C *spec = G.spec;
+    auto pick = [&](int g) {
+        G.gs = G.gp = d.grid + g * ng;
+        G.spec = spec + (size_t)g * G.K0 * n;
+    };
+    for (int t = blockIdx.x; t < ngrid * G.K0; t += gridDim.x) {
+        pick(t / G.K0);
+        plane_forward<LT, false>(G, lp, s_ax, t % G.K0, tid);
+    }
+    grid.sync();
+    for (int t = blockIdx.x; t < ngrid * tiles; t += gridDim.x) {
+        pick(t / tiles);
+        columns<LT>(G, lp, s_ax, t % tiles, tid);
+    }
+    grid.sync();
+    for (int t = blockIdx.x; t < ngrid * G.K0; t += gridDim.x) {
+        pick(t / G.K0);
+        plane_inverse<LT>(G, lp, s_ax, t % G.K0, tid);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1039,6 +1091,40 @@ bool fft_axis(FftAxis &A, int n, int tw, bool fp64) {
     return rest == 1;
 }
 
+// Transform part of a plan for `blocks` blocks: the axes' passes, buffer size
+// and index reciprocals; false for sizes with other primes or above 128.
+template <typename R>
+bool fft_plan(LoopPlan &L, const int K[3], int blocks) {
+    for (int c = 0; c < 3; ++c) {
+        if (K[c] > 128 || !fft_axis(L.ax[c], K[c], L.ntw, sizeof(R) == 8)) return false;
+        L.ntw += K[c];
+    }
+    const int nz = K[2] / 2 + 1, n = K[1] * nz, lines = (K[1] + 1) / 2;
+    L.xt = std::max(4, (n + blocks - 1) / blocks);
+    L.nbuf = std::max(std::max(K[2] * (lines | 1), n), K[0] * L.xt);
+    L.div_k2 = recip(K[2]);
+    L.div_l = recip(lines);
+    L.div_nz = recip(nz);
+    L.div_xt = recip(L.xt);
+    return true;
+}
+
+// whether a block of kernel f with smem bytes of dynamic shared memory fits an SM
+bool fits(const void *f, size_t smem) {
+    int dev = 0, most = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, f) != cudaSuccess || smem + fa.sharedSizeBytes > (size_t)most) return false;
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, LT, smem) != cudaSuccess || per_sm < 1) {
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+
 }  // namespace
 
 // ncta stays 0 for what the kernel does not take: larger systems (above
@@ -1054,33 +1140,36 @@ void loop_plan(LoopPlan &L, int M, int periodic, const int K[3], int tls, int n_
     // rows and chunks of the list start on 16-byte boundaries and whole chunks stay inside a row
     L.staged = tls % CH<R> == 0;
     const int ncta = (M + L.mper - 1) / L.mper;
-    if (periodic) {
-        for (int c = 0; c < 3; ++c) {
-            if (K[c] > 128 || !fft_axis(L.ax[c], K[c], L.ntw, sizeof(R) == 8)) return;
-            L.ntw += K[c];
-        }
-        const int nz = K[2] / 2 + 1, n = K[1] * nz, lines = (K[1] + 1) / 2;
-        L.xt = std::max(4, (n + ncta - 1) / ncta);
-        L.nbuf = std::max(std::max(K[2] * (lines | 1), n), K[0] * L.xt);
-        L.div_k2 = recip(K[2]);
-        L.div_l = recip(lines);
-        L.div_nz = recip(nz);
-        L.div_xt = recip(L.xt);
-    }
+    if (periodic && !fft_plan<R>(L, K, ncta)) return;
     L.smem = loop_mem<R>(L.mper, periodic, L.ntw, L.nbuf, L.staged).total;
-    int dev = 0, most = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     const void *f = periodic ? (const void *)k_pcg_loop<R, true> : (const void *)k_pcg_loop<R, false>;
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, f) != cudaSuccess || L.smem + fa.sharedSizeBytes > (size_t)most) return;
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, LT, L.smem) != cudaSuccess || per_sm < 1) {
-        cudaGetLastError();
-        return;
-    }
-    L.ncta = ncta;
+    if (fits(f, L.smem)) L.ncta = ncta;
+}
+
+template <typename R>
+void conv_plan(LoopPlan &L, const int K[3], int n_sm) {
+    L.ncta = 0;
+    L.nbuf = L.ntw = 0;
+    if (n_sm < 1 || !fft_plan<R>(L, K, n_sm)) return;
+    const size_t c = sizeof(typename Cplx<R>::T);
+    L.smem = ((L.ntw * c + 15) & ~(size_t)15) + 2 * L.nbuf * c;
+    if (fits((const void *)k_grid_conv<R>, L.smem)) L.ncta = n_sm;
+}
+
+template <typename R>
+cudaError_t launch_grid_conv(const KParams &p, DevState<R> &d, const LoopPlan &lp, int ngrid, Launch L) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)lp.ncta);
+    cfg.blockDim = dim3(LT);
+    cfg.dynamicSmemBytes = lp.smem;
+    cfg.stream = L.s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    count(L);
+    return cudaLaunchKernelEx(&cfg, k_grid_conv<R>, p, d, lp, ngrid);
 }
 
 std::vector<double> loop_twiddles(const int K[3]) {
@@ -1124,7 +1213,10 @@ cudaError_t launch_pcg_cluster(const KParams &p, DevState<float> &d, int nmax, i
 }
 
 #define INST(R)                                                                                              \
-    template void loop_plan<R>(LoopPlan &, int, int, const int *, int, int);                                    \
+    template void loop_plan<R>(LoopPlan &, int, int, const int *, int, int);                                 \
+    template void conv_plan<R>(LoopPlan &, const int *, int);                                                \
+    template cudaError_t launch_grid_conv<R>(const KParams &, DevState<R> &, const LoopPlan &, int, Launch); \
+                                    \
     template cudaError_t launch_pcg_loop<R>(const KParams &, DevState<R> &, const LoopPlan &, const MuGuess &, int, \
                                             double *, Launch);
 INST(float)

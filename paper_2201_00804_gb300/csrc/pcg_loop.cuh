@@ -47,6 +47,11 @@ struct LoopPlan {
 // Fills the plan's sizes for M molecules (grid K when periodic); ncta stays 0
 // when the kernel does not take the problem.
 template <typename R> void loop_plan(LoopPlan &L, int M, int periodic, const int K[3], int tls, int n_sm);
+// Plan of the one-kernel grid convolution (transform fields only); ncta stays
+// 0 for grids it does not take, which go through the transform library.
+template <typename R> void conv_plan(LoopPlan &L, const int K[3], int n_sm);
+template <typename R>
+cudaError_t launch_grid_conv(const KParams &p, DevState<R> &d, const LoopPlan &lp, int ngrid, Launch L);
 // twiddles of all axes, re/im interleaved
 std::vector<double> loop_twiddles(const int K[3]);
 template <typename R>

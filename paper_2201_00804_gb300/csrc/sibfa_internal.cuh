@@ -186,6 +186,7 @@ struct DevState {
     // x -> (I + eps) x of atoms and cell, and the reciprocal-space parts
     double *vir;        // M*9
     double *vir_r;      // M*9 (reciprocal chain)
+    double *vir_s;      // M*9 (short-range kernels)
     double *virk;       // 2 passes x VK_BLOCKS x 8: k-space sums per convolution block
     void *qhat_p;       // K0*K1*(K2/2+1) complex: spectrum of the permanent grid (kept for the force pass)
     R *vphi;            // M*9 gradient of the reciprocal permanent potential at O, H1, H2
@@ -848,11 +849,12 @@ inline DevState<R> rec_view(const DevState<R> &d) {
     r.vir = d.vir_r;
     return r;
 }
-// the short-range kernels' view: their own point-gradient array
+// the short-range kernels' view: their own point-gradient and virial arrays
 template <typename R>
 inline DevState<R> short_view(const DevState<R> &d) {
     DevState<R> r = d;
     r.gpt = d.gpt_s;
+    r.vir = d.vir_s;
     return r;
 }
 
