@@ -562,7 +562,7 @@ __host__ __device__ inline LoopMem loop_mem(int mper, int periodic, int ntw, int
 }
 
 template <typename R, bool PER>
-__global__ void __launch_bounds__(LT, sizeof(R) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(LT, 2)
     k_pcg_loop(KParams p, DevState<R> d, LoopPlan lp, MuGuess guess, int warm, double *push) {
     using C = typename Cplx<R>::T;
     unsigned char *raw = loop_raw;
@@ -860,7 +860,7 @@ __global__ void __launch_bounds__(LT, sizeof(R) == 4 ? 2 : 1)
 // each at these sizes (55 us in FP64 at 24^3).
 // ---------------------------------------------------------------------------
 template <typename R>
-__global__ void __launch_bounds__(LT, sizeof(R) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(LT, 2)
     k_grid_conv(KParams p, DevState<R> d, LoopPlan lp, int ngrid) {
     using C = typename Cplx<R>::T;
     namespace cg = cooperative_groups;
