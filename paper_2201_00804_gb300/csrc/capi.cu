@@ -236,6 +236,11 @@ sibfa_status alloc_state(sibfa_ctx *ctx, DevState<R> &d) {
     }
     AL(d.ctin, M * 8);
     AL(d.spk, M * 20);
+    // Inbox rows of the short-range pairs: in a box half the list's capacity (a molecule owns about half of its
+    // pairs; more rows than that are added directly), in the gas phase one a neighbour and part
+    d.in_rows = ctx->opts.periodic ? MAXN / 2 : (sizeof(R) == 4 ? 1 : 2) * (ctx->kp.tls / 3);
+    AL(d.inbox, (size_t)M * d.in_rows * (ctx->opts.periodic ? 16 : 24));
+    AL(d.inn, M);
     AL(d.epart, M * NTERM);
     AL(d.epw, M * NS * 2);
     AL(d.vir, M * 9);
@@ -309,12 +314,26 @@ sibfa_status alloc_state(sibfa_ctx *ctx, DevState<R> &d) {
 template <typename R>
 void fill_scal(Scal<R> &s, const KParams &k) {
     s.rc2 = R(k.rc2); s.alpha = R(k.alpha); s.thole = R(k.thole);
-    s.cs_o = R(k.cs_o); s.cp_o = R(k.cp_o); s.cs_h = R(k.cs_h); s.cp_h = R(k.cp_h);
     s.cs_lp = R(k.cs_lp); s.cp_lp = R(k.cp_lp); s.g_o = R(k.g_o); s.g_h = R(k.g_h);
     s.inv_nval_o = R(1.0 / k.nval_o); s.inv_nval_h = R(1.0 / k.nval_h);
-    s.rep_f = R(k.rep_f); s.rep_c1 = R(k.rep_c1); s.rep_c2 = R(k.rep_c2); s.occ = R(k.occ); s.nlp = R(k.nlp);
-    s.c6 = R(k.c6); s.c8 = R(k.c8); s.c10 = R(k.c10); s.g6 = R(k.g6); s.g8 = R(k.g8); s.g10 = R(k.g10);
-    s.delta = R(k.delta); s.xd_c1 = R(k.xd_c1); s.xd_c2 = R(k.xd_c2); s.xd_c3 = R(k.xd_c3);
+    s.rep_c1 = R(k.rep_c1); s.rep_c2 = R(k.rep_c2); s.occ = R(k.occ); s.nlp = R(k.nlp);
+    s.g6 = R(k.g6); s.g8 = R(k.g8); s.g10 = R(k.g10);
+    const double cs[3] = {k.cs_o, k.cs_h, k.cs_lp}, cp[3] = {k.cp_o, k.cp_h, k.cp_lp};
+    const double cn[3] = {k.c6, k.c8, k.c10}, beta[3] = {k.beta[0], k.beta[1], k.beta[3]};
+    for (int a = 0; a < 3; ++a)
+        for (int b = 0; b < 3; ++b) {
+            // the p-p factor of a bond with a lone pair is rep_f
+            const double pp = (a == 2) != (b == 2) ? k.rep_f : 2.0;
+            s.rep_o[a][b][0] = R(cs[a] * cs[b]);
+            s.rep_o[a][b][1] = R(k.rep_f * cp[a] * cs[b]);
+            s.rep_o[a][b][2] = R(k.rep_f * cs[a] * cp[b]);
+            s.rep_o[a][b][3] = R(pp * cp[a] * cp[b]);
+            const int lone = (a == 2) + (b == 2);
+            const double pref[3] = {-beta[a] * beta[b], -0.5 * k.delta, -0.25 * k.nlp * k.nlp};
+            const double xc[3] = {k.xd_c1, 0.5 * k.nlp * k.xd_c3, 0.25 * k.nlp * k.nlp * k.xd_c2};
+            for (int n = 0; n < 3; ++n) s.disp_c[n][a][b] = R(pref[lone] * cn[n] * pow(k.disp_km[a][b].d, -6.0 - 2.0 * n));
+            s.xd_c[a][b] = R(xc[lone] * beta[a] * beta[b]);
+        }
     s.ct_t = R(k.ct_t); s.ct_m = R(k.ct_m); s.ct_ae = R(k.ct_ae); s.ct_ah = R(k.ct_ah);
     for (int c = 0; c < 3; ++c) s.kl[c] = k.box[c] > 0 ? R((double)k.K[c] / k.box[c]) : R(0);
     s.ike = R(1.0 / k.ke);
@@ -911,7 +930,7 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
         DevState<R> ds = short_view(d);
         // resident blocks per SM (0: uncapped), chosen by the autotuner: a cap
         // leaves every SM registers for the solve's small kernels
-        launch_short(p, ds, Launch{ctx->s3, &ctx->launches}, 0, short_cap(ctx));
+        launch_short(p, ds, Launch{ctx->s3, &ctx->launches}, short_cap(ctx));
     }
     // mixed periodic path: the FP64 intramolecular Ewald energy, beside everything else
     if (sizeof(R) == 4 && p.periodic && !dipoles_only)

@@ -29,9 +29,12 @@ enum { F_CUTOFF = 1, F_NEIGHBOR = 2, F_CTDEN = 4, F_NAN = 8, F_NOCONV = 16, F_TI
 template <typename R>
 struct Scal {
     R rc2, alpha, thole;
-    R cs_o, cp_o, cs_h, cp_h, cs_lp, cp_lp, g_o, g_h, inv_nval_o, inv_nval_h;
-    R rep_f, rep_c1, rep_c2, occ, nlp;
-    R c6, c8, c10, g6, g8, g10, delta, xd_c1, xd_c2, xd_c3;
+    R cs_lp, cp_lp, g_o, g_h, inv_nval_o, inv_nval_h;
+    R rep_c1, rep_c2, occ, nlp;
+    R g6, g8, g10;
+    R rep_o[3][3][4];     // overlap A + B cx + C cy + D cx cy of centres of two kinds (O, H, lone pair)
+    R disp_c[3][3][3];    // C_n prefactors of two kinds, n = 6, 8, 10, of 1/r^n
+    R xd_c[3][3];         // exchange-dispersion prefactors of two kinds
     R ct_t, ct_m, ct_ae, ct_ah;
     R kl[3];   // SPME grid points per unit length, K / L
     R ike;     // 1 / ke
@@ -214,6 +217,9 @@ struct DevState {
     R *lamaR, *cvs;
     R *ctin;            // M*8 working-precision charge-transfer inputs (V_lp, V_int, V(a))
     R *spk;             // M*20 short-range point data (offset from O, valence factor) x 5 points
+    R *inbox;           // M*in_rows rows of short-range gradients from the pairs others own (gas phase: all pairs)
+    int *inn;           // M rows in use (periodic)
+    int in_rows;        // rows a molecule has
     int *tl_n, *tl_j;                   // polarization pair list: count per atom; partner | sgn(g2) << 31
     R *tl_x, *tl_y, *tl_z, *tl_g1;      // sqrt|g2| x (x the pair displacement) and g1
     double *partial;    // reduction partials
@@ -822,8 +828,7 @@ template <typename R> void launch_sites(const KParams &p, DevState<R> &d, double
 template <typename R> void launch_neighbors(const KParams &p, DevState<R> &d, int ncell[3], Launch L);
 template <typename R> void launch_real_perm(const KParams &p, DevState<R> &d, Launch L);
 template <typename R> void launch_lp_potential(const KParams &p, DevState<R> &d, Launch L);
-template <typename R> void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_blocks = 0,
-                                         int max_per_sm = 0);
+template <typename R> void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm = 0);
 template <typename R> void launch_ct(const KParams &p, DevState<R> &d, Launch L);
 template <typename R> void launch_intra_perm(const KParams &p, DevState<R> &d, Launch L);
 template <typename R> void launch_real_tmu(const KParams &p, DevState<R> &d, double *out,
