@@ -106,12 +106,35 @@ struct PermT {
 // For gas-phase clusters this brings the FP32 multipole energy some 30x
 // closer to FP64 than summing the site-pair energies directly.
 //
+// What depends on the target site and the source molecule alone (y2, its
+// products with the target, y0) is formed once for the molecule's five sources.
+//
 // ms: source multipole of site s_ (quadrupole / 3).  At a polarizable target
 // x, T2 and g1 return the pair's entry of the polarization matrix (field of a
 // dipole mu at x: T2 (mu.x) x + g1 mu).
+template <typename R>
+struct GasRef {
+    V3<R> y2, Tty;       // x_t - O_j, (Theta_t / 3) y2
+    R b2, r2, mu, yTy;   // 1/|y2|, |y2|, mu_t.y2, y2.Theta_t.y2
+    R b0, r0;            // 1/|D|, |D|
+    __device__ __forceinline__ GasRef(const PermT<R> &T, V3<R> D) {
+        y2 = T.o - D;
+        const R yy = dot(y2, y2), DD = dot(D, D);
+        b2 = rsqrt_(yy);
+        r2 = yy * b2;
+        Tty = symv(T.m.th, y2);
+        mu = dot(T.m.mu, y2);
+        yTy = R(3.0) * dot(y2, Tty);
+        b0 = rsqrt_(DD);
+        r0 = DD * b0;
+    }
+    __device__ __forceinline__ GasRef() {}
+};
+
 template <typename R, bool PER, bool ATOM_SRC, bool VIR>
-__device__ __forceinline__ void perm_pair(const KParams &p, const PermT<R> &T, const Mp<R> &ms, int s_, V3<R> rv,
-                                          V3<R> osrc, PermAcc<R> &acc, R &g1, R &T2, V3<R> &x) {
+__device__ __forceinline__ void perm_pair(const KParams &p, const PermT<R> &T, const GasRef<R> &G, const Mp<R> &ms,
+                                          int s_, V3<R> rv, V3<R> osrc, bool energy, PermAcc<R> &acc, R &g1, R &T2,
+                                          V3<R> &x) {
     const Scal<R> &S = sc<R>(p);
     const bool atom = T.w < 3;
     const R m1 = R(-1.0), two = R(2.0);
@@ -131,16 +154,15 @@ __device__ __forceinline__ void perm_pair(const KParams &p, const PermT<R> &T, c
     const R pdt = symdd(s.th, t.th);
     Field2<R> F;
     const V3<R> gel = pair_grad(t, s, x, B, pdt, F);
-    R U;
+    R U = R(0);
     if (PER) {
         U = t.q * (s.q * B[0] + s.s * B[1] + s.w * B[2]) + dot(t.mu, F.d1) + F.Rr * t.w + two * dot(t.p, F.U) +
             two * B[2] * pdt;
-    } else {
+    } else if (energy) {
         const R three = R(3.0);
         const R a = rinv, a3 = a * r2i, a5 = a3 * r2i;
         // charge-charge, reference -D
-        const R RR = dot(rv, rv), b0 = rsqrt_<R>(RR);
-        U = t.q * s.q * ((two * dot(sv, rv) - dot(sv, sv)) * a * b0 / (r + RR * b0));
+        U = t.q * s.q * ((two * dot(sv, rv) - dot(sv, sv)) * a * G.b0 / (r + G.r0));
         // target charge, reference O_i - x_s
         const V3<R> y1 = m1 * (rv + osrc);
         const R y1y1 = dot(y1, y1), b1 = rsqrt_<R>(y1y1);
@@ -154,17 +176,16 @@ __device__ __forceinline__ void perm_pair(const KParams &p, const PermT<R> &T, c
             U += T.Q * (mu_y1 * b13 + y1Ty1 * b13 * b1 * b1);
         }
         // source charge, reference x_t - O_j
-        const V3<R> y2 = T.o - rv;
-        const R y2y2 = dot(y2, y2), b2 = rsqrt_<R>(y2y2);
-        ref_diff35(two * dot(y2, osrc) - dot(osrc, osrc), a, b2, r, y2y2 * b2, D3, D5);
-        const V3<R> Tto = symv(t.th, osrc), Tty = symv(t.th, y2);
-        U += s.q * (dot(t.mu, osrc) * a3 - dot(t.mu, y2) * D3 + three * (dot(osrc, Tto) - two * dot(y2, Tto)) * a5 +
-                    three * dot(y2, Tty) * D5);
+        ref_diff35(two * dot(G.y2, osrc) - dot(osrc, osrc), a, G.b2, r, G.r2, D3, D5);
+        const V3<R> Tto = symv(t.th, osrc);
+        U += s.q * (dot(t.mu, osrc) * a3 - G.mu * D3 + three * (dot(osrc, Tto) - two * dot(osrc, G.Tty)) * a5 +
+                    G.yTy * D5);
         // target dipole and quadrupole in the source dipole and quadrupole field
         U += dot(t.mu, s.grad_mp(x, B[1], B[2], B[3])) + (s.s * B[3] + s.w * B[4]) * t.w + two * dot(t.p, F.U) +
              two * B[2] * pdt;
     }
-    acc.Ue.add(R(0.5) * U);
+    if (PER) acc.Ue.add(R(0.5) * U);
+    else if (energy) acc.Ue.add(U);
     V3<R> g = gel;
     acc.gm = acc.gm + F.d1;
     symacc(acc.gt, F.d2);
@@ -211,7 +232,8 @@ __device__ __forceinline__ void perm_pair(const KParams &p, const PermT<R> &T, c
             g = g + f1 * s.mu + c * s.v;
         }
         g = g - gq * x;
-        acc.Up.add(R(0.5) * pen);
+        if (PER) acc.Up.add(R(0.5) * pen);
+        else if (energy) acc.Up.add(pen);
     }
     acc.gr = acc.gr + g;
     if (VIR) vir_add(acc.W, g, x, R(0.5));
@@ -227,13 +249,101 @@ __device__ __forceinline__ void perm_pair(const KParams &p, const PermT<R> &T, c
     }
 }
 
-// Blocks per SM, FP32: periodic 18 (112 registers; 32,000 waters: 1728 us,
+// An entry of the polarization matrix T: the field of a dipole mu at x is
+// T2 (mu.x) x + g1 mu = sgn(T2) (mu.y) y + g1 mu with y = sqrt|T2| x: four
+// values and the sign in the index's top bit.
+template <typename R>
+__device__ __forceinline__ void store_tpair(const DevState<R> &d, size_t te, int atom, V3<R> x, R T2, R g1) {
+    const R sq = sqrt_(fabs(T2));
+    d.tl_j[te] = atom | (T2 < R(0) ? int(0x80000000u) : 0);
+    d.tl_x[te] = sq * x.x;
+    d.tl_y[te] = sq * x.y;
+    d.tl_z[te] = sq * x.z;
+    d.tl_g1[te] = g1;
+}
+
+// Gas phase: the list entries of consecutive molecules (at most 32) on one
+// side of the ownership of pairs, 32 at a time in order.  Molecule i of a
+// cluster [lo, hi) owns its pairs with the lower ones of its parity and the
+// higher ones of the other; its list holds all of the cluster but itself.  A molecule
+// without entries takes one place.
+constexpr int GAS_BLOCKS = 16;   // one-warp blocks an SM, FP32
+struct GasWalk {
+    int first, n_mol, others;   // molecules; 0: the owned entries, 1: the rest
+    int nl, ll;                 // lane k's: entries of molecule first + k, and the molecules below it in its cluster
+    int m = 0, at = 0;          // next molecule and entry
+    int mol, slot;              // this lane's: molecule (-1: idle) and list place (-1: none)
+    int n_used;
+    template <typename R>
+    __device__ GasWalk(const KParams &p, const DevState<R> &d, int mpw, int lane)
+        : first(blockIdx.x * mpw), n_mol(min(mpw, p.M - first)), others(blockIdx.z) {
+        nl = ll = 0;
+        if (lane < n_mol) {
+            const int nn = d.nnbr[first + lane];
+            ll = min(first + lane - d.cl_start[d.cl_of[first + lane]], nn);   // (a list that overflowed is flagged)
+            const int up = nn - ll;
+            nl = others ? (ll + 1) / 2 + up / 2 : ll / 2 + (up + 1) / 2;
+        }
+    }
+    __device__ bool next(int lane) {
+        mol = slot = -1;
+        n_used = 0;
+        while (n_used < 32 && m < n_mol) {
+            const int n = __shfl_sync(0xffffffffu, nl, m), lo = __shfl_sync(0xffffffffu, ll, m);
+            const int places = max(n, 1), take = min(32 - n_used, places - at);
+            if (lane >= n_used && lane < n_used + take) {
+                mol = first + m;
+                if (n > 0) {
+                    const int k = at + lane - n_used, below = others ? (lo + 1) / 2 : lo / 2;
+                    // below: lo - 1 - others.. downwards by twos; above (places shift by one, i is not listed) upwards
+                    slot = k < below ? lo - 2 * (k + 1) + others : lo + 2 * (k - below) + others;
+                }
+            }
+            n_used += take;
+            at += take;
+            if (at == places) ++m, at = 0;
+        }
+        return n_used > 0;
+    }
+    // f(molecule, lanes from, to, whether these hold the molecule's first entry)
+    template <typename F>
+    __device__ void segments(bool start_new, F f) const {
+        int k = 0;
+        for (int c = 0; c < n_used; ++k) {
+            const int g = __shfl_sync(0xffffffffu, mol, c);
+            const int n = __popc(__ballot_sync(0xffffffffu, mol == g));
+            f(g, c, c + n, k > 0 || start_new);
+            c += n;
+        }
+    }
+};
+// sum over columns c0 <= c < c1 of row lane (< nv) of buf (33 a row); FP32: compensated
+template <typename R>
+__device__ __forceinline__ double segment_sum(const R *buf, int lane, int nv, int c0, int c1) {
+    if (lane >= nv) return 0.0;
+    Acc<R> a;
+    R s = R(0);
+    for (int c = c0; c < c1; ++c) {
+        if (sizeof(R) == 4) a.add(buf[lane * 33 + c]);
+        else s += buf[lane * 33 + c];
+    }
+    return sizeof(R) == 4 ? a.get() : double(s);
+}
+// Molecules a warp of k_perm_gas: whole rounds in FP32 (4096 clusters of 17
+// waters: 1318 us at 2, 1234 at 4, 1154 at 8, 1113 at 32); in FP64, bound by
+// the pipe of each quarter of an SM, few, which spreads the work (824 waters: 510 us at 4, 570 at 8, 802 at 16).
+template <typename R>
+int gas_mpw(const KParams &p) {
+    return warp_molecules(p.M, 0.5 * (p.M / (double)p.n_cl - 1.0), 2 * NS, (sizeof(R) == 4 ? GAS_BLOCKS : 4), 0.25,
+                          sizeof(R) == 4 ? 32 : 4);
+}
+
+// Boxes.  Blocks per SM, FP32: 18 (112 registers; 32,000 waters: 1728 us,
 // 1909 at 16, 1735 at 20, where registers spill, 1926 with the five sites in
-// one block), gas phase 17 (4096 clusters: 1409 us, 1423 at 18, 1444 before);
-// FP64 8 (216 waters: 274 us against 416 in one block).
-template <typename R, bool PER, bool VIR>
+// one block); FP64 8 (216 waters: 274 us against 416 in one block).
+template <typename R, bool VIR>
 __global__ void __launch_bounds__(VIR ? 32 * NS : 32,
-                                  VIR ? (sizeof(R) == 4 ? 3 : 2) : (sizeof(R) == 4 ? (PER ? 18 : 17) : 8))
+                                  VIR ? (sizeof(R) == 4 ? 3 : 2) : (sizeof(R) == 4 ? 18 : 8))
     k_real_perm(KParams p, DevState<R> d) {
     constexpr int NW = VIR ? NS : 1;   // warps a block: the virial variant sums the sites' in a fixed order
     __shared__ double s_w[VIR ? NW : 1][9];
@@ -244,10 +354,8 @@ __global__ void __launch_bounds__(VIR ? 32 * NS : 32,
     const int w = VIR ? wq : blockIdx.x % NS;   // target site
     PairQueue<R> &q = qs[wq];
     const Mp<R> mt = load_mp(d.gmp + (i * NS + w) * GMP);
-    R Qi = R(0);   // gas phase: charge of molecule i (remainders of the reference-difference energy, see perm_pair)
-    if (!PER)
-        for (int s = 0; s < NS; ++s) Qi += d.gmp[(i * NS + s) * GMP];
-    const PermT<R> T{scaled(mt, R(1.0 / 3.0)), my_pt(d, i, w), zsite<R>(p, w) - mt.q, Qi, w};
+    const PermT<R> T{scaled(mt, R(1.0 / 3.0)), my_pt(d, i, w), zsite<R>(p, w) - mt.q, R(0), w};
+    const GasRef<R> none;
     const R rc2 = sc<R>(p).rc2;
     const size_t tbase = (size_t)(i * 3 + (w < 3 ? w : 0)) * p.tls;   // T-pair list of target atom w
 
@@ -263,21 +371,10 @@ __global__ void __launch_bounds__(VIR ? 32 * NS : 32,
         constexpr bool AT = decltype(atom_src)::value;
         const int js = q.js[e], j = js >> 3, s = js & 7;
         const Mp<R> ms = scaled(load_mp_g(d.gmp + (j * NS + s) * GMP), R(1.0 / 3.0));
-        V3<R> os = mk(R(0), R(0), R(0)), x;
-        if (!PER) os = my_pt(d, j, s);
+        V3<R> x;
         R g1 = R(0), T2 = R(0);
-        perm_pair<R, PER, AT, VIR>(p, T, ms, s, q.at(e), os, acc, g1, T2, x);
-        if (AT && w < 3 && p.tlist) {
-            // the same atom pair in the polarization matrix T: the field of a
-            // dipole mu at x is T2 (mu.x) x + g1 mu = sgn(T2) (mu.y) y + g1 mu
-            // with y = sqrt|T2| x: four values and the sign in the index's top bit
-            const R sq = sqrt_(fabs(T2));
-            d.tl_j[te] = (j * 3 + s) | (T2 < R(0) ? int(0x80000000u) : 0);
-            d.tl_x[te] = sq * x.x;
-            d.tl_y[te] = sq * x.y;
-            d.tl_z[te] = sq * x.z;
-            d.tl_g1[te] = g1;
-        }
+        perm_pair<R, true, AT, VIR>(p, T, none, ms, s, q.at(e), T.o, true, acc, g1, T2, x);
+        if (AT && w < 3 && p.tlist) store_tpair(d, te, j * 3 + s, x, T2, g1);
     };
 
     int ha = 0, ta = 0, hm = 0, tm = 0;   // queue heads and tails (warp-uniform, monotone)
@@ -297,19 +394,7 @@ __global__ void __launch_bounds__(VIR ? 32 * NS : 32,
             for (int s = 0; s < NS; ++s) {
                 rs[s] = dO + mk(__ldg(offj + s * 3), __ldg(offj + s * 3 + 1), __ldg(offj + s * 3 + 2));
                 const V3<R> x = T.o - rs[s];
-                if (!PER || dot(x, x) < rc2) bits |= 1u << s;
-                if (!PER) rs[s] = dO;   // queued: the O-O displacement (see perm_pair)
-            }
-            if (!PER) {
-                R Qj = R(0);
-                for (int s = 0; s < NS; ++s) Qj += d.gmp[(j * NS + s) * GMP];
-                // Q_j times the reference value of the target's terms: the
-                // charge-charge one (O target only) and the dipole/quadrupole ones
-                const V3<R> y2 = T.o - dO;
-                const R b2 = rsqrt_(dot(y2, y2)), b23 = b2 * b2 * b2;
-                R rem = R(3) * dot(y2, symv(T.m.th, y2)) * b23 * b2 * b2 - dot(T.m.mu, y2) * b23;
-                if (w == 0) rem += Qi * rsqrt_(dot(dO, dO));
-                acc.Ue.add(R(0.5) * Qj * rem);
+                if (dot(x, x) < rc2) bits |= 1u << s;
             }
         }
         int na, nm;
@@ -366,14 +451,104 @@ __global__ void __launch_bounds__(VIR ? 32 * NS : 32,
     }
 }
 
+// Gas phase: no cutoff, so no queue.  The lists of mpw consecutive molecules
+// are taken one after another, 32 entries (target molecule, source molecule)
+// a round; a lane evaluates the five sources of its entry in turn at target
+// site w = blockIdx.y, and the entries of each molecule are then summed.  The
+// energy, a quarter of the work here (see perm_pair), is the same from both
+// sides of a pair: it is taken from the entries that own their pair (blockIdx.z
+// = 0), and the others skip it.  Bound by issue and latency at 16 warps an SM (127
+// registers; 14: 1152 us).  4096 clusters of 17 waters 1282 -> 1113 us, 824
+// waters in FP64 clusters 600 -> 510 us, against a warp per target site with queues.
+template <typename R, bool VIR>
+__global__ void __launch_bounds__(32, sizeof(R) == 4 ? GAS_BLOCKS : 8) k_perm_gas(KParams p, DevState<R> d, int mpw) {
+    constexpr int NV = 19 + (VIR ? 9 : 0);
+    __shared__ R buf[NV * 33];
+    const int lane = threadIdx.x, w = blockIdx.y;
+    const bool energy = blockIdx.z == 0;
+    GasWalk walk(p, d, mpw, lane);
+    for (bool fresh = true; fresh = walk.at == 0, walk.next(lane);) {
+        PermAcc<R> acc;
+        acc.gr = mk(R(0), R(0), R(0));
+        acc.gm = acc.gr;
+        acc.ef = acc.gr;
+        acc.gt = Sym<R>{};
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc.W[k] = R(0);
+        const int i = walk.mol, slot = walk.slot;
+        if (i >= 0 && slot >= 0) {
+            const int j = d.nbr[i * MAXN + slot];
+            const R *dp = d.ndo + ((size_t)i * MAXN + slot) * 3;
+            const V3<R> D = mk(dp[0], dp[1], dp[2]);
+            const Mp<R> mt = load_mp_g(d.gmp + (i * NS + w) * GMP);
+            R Qi = R(0), Qj = R(0);   // molecule charges (remainders, see perm_pair)
+            if (w == 0 && energy)
+                for (int s = 0; s < NS; ++s) Qi += d.gmp[(i * NS + s) * GMP];
+            const PermT<R> T{scaled(mt, R(1.0 / 3.0)), my_pt(d, i, w), zsite<R>(p, w) - mt.q, Qi, w};
+            const GasRef<R> G(T, D);
+            const size_t te = (size_t)(i * 3 + (w < 3 ? w : 0)) * p.tls + slot * 3;
+            auto eval = [&](auto atom_src, int s) {
+                constexpr bool AT = decltype(atom_src)::value;
+                const Mp<R> m = load_mp_g(d.gmp + (j * NS + s) * GMP);
+                Qj += m.q;
+                V3<R> x;
+                R g1 = R(0), T2 = R(0);
+                perm_pair<R, false, AT, VIR>(p, T, G, scaled(m, R(1.0 / 3.0)), s, D, my_pt(d, j, s), energy, acc, g1,
+                                              T2, x);
+                if (AT && w < 3 && p.tlist) store_tpair(d, te + s, j * 3 + s, x, T2, g1);
+            };
+#pragma unroll 1
+            for (int s = 0; s < 3; ++s) eval(std::true_type{}, s);
+#pragma unroll 1
+            for (int s = 3; s < NS; ++s) eval(std::false_type{}, s);
+            // Q_j times the reference values of the target's terms: the
+            // dipole/quadrupole ones and (O target only) the charge-charge one
+            if (energy) {
+                const R b23 = G.b2 * G.b2 * G.b2;
+                R rem = G.yTy * b23 * G.b2 * G.b2 - G.mu * b23;
+                if (w == 0) rem += Qi * G.b0;
+                acc.Ue.add(Qj * rem);
+            }
+        }
+        const R vals[19] = {acc.gr.x, acc.gr.y, acc.gr.z, acc.gm.x, acc.gm.y, acc.gm.z, acc.gt.xx,
+                            acc.gt.yy, acc.gt.zz, acc.gt.xy, acc.gt.xz, acc.gt.yz, acc.ef.x, acc.ef.y,
+                            acc.ef.z, acc.Ue.hi, acc.Ue.lo, acc.Up.hi, acc.Up.lo};
+#pragma unroll
+        for (int k = 0; k < NV; ++k) buf[k * 33 + lane] = k < 19 ? vals[k < 19 ? k : 0] : acc.W[k < 19 ? 0 : k - 19];
+        __syncwarp();
+        const double ke = p.ke;
+        walk.segments(fresh, [&](int m, int c0, int c1, bool first) {
+            const double t = segment_sum<R>(buf, lane, NV, c0, c1);
+            double *dst = nullptr;
+            if (lane < 3) dst = d.gpt + (m * NP + w) * 3 + lane;
+            else if (lane < 6) dst = d.gmu + (m * NS + w) * 3 + lane - 3;
+            else if (lane < 12) dst = d.gth + (m * NS + w) * 6 + lane - 6;
+            else if (lane < 15 && w < 3) dst = d.efield + m * 9 + w * 3 + lane - 12;
+            if (dst) atomicAdd(dst, (lane < 6 ? ke : (lane < 12 ? ke * (1.0 / 3.0) : 1.0)) * t);
+            // per-site energies (summed over the five sites in a fixed order by k_pol_energy)
+            const double e = ke * (t + __shfl_down_sync(0xffffffffu, t, 1));
+            if (energy && (lane == 15 || lane == 17)) {
+                double *o = d.epw + (m * NS + w) * 2 + (lane == 17);
+                *o = first ? e : *o + e;
+            }
+            if (VIR && lane >= 19 && lane < NV) atomicAdd(d.vir + m * 9 + lane - 19, ke * t);
+            if (energy && w < 3 && lane == 0 && first) d.tl_n[m * 3 + w] = 3 * d.nnbr[m];
+        });
+        __syncwarp();
+    }
+}
+
 template <typename R>
 void launch_real_perm(const KParams &p, DevState<R> &d, Launch L) {
-    if (p.vir) {
-        if (p.periodic) k_real_perm<R, true, true><<<p.M, 32 * NS, 0, L.s>>>(p, d);
-        else k_real_perm<R, false, true><<<p.M, 32 * NS, 0, L.s>>>(p, d);
+    if (!p.periodic) {
+        const int mpw = gas_mpw<R>(p);
+        const dim3 g((unsigned)((p.M + mpw - 1) / mpw), NS, 2);
+        if (p.vir) k_perm_gas<R, true><<<g, 32, 0, L.s>>>(p, d, mpw);
+        else k_perm_gas<R, false><<<g, 32, 0, L.s>>>(p, d, mpw);
+    } else if (p.vir) {
+        k_real_perm<R, true><<<p.M, 32 * NS, 0, L.s>>>(p, d);
     } else {
-        if (p.periodic) k_real_perm<R, true, false><<<p.M * NS, 32, 0, L.s>>>(p, d);
-        else k_real_perm<R, false, false><<<p.M * NS, 32, 0, L.s>>>(p, d);
+        k_real_perm<R, false><<<p.M * NS, 32, 0, L.s>>>(p, d);
     }
     count(L);
 }

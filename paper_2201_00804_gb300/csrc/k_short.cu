@@ -727,9 +727,8 @@ __global__ void __launch_bounds__(128) k_short_gather(KParams p, DevState<R> d, 
 // kernels of the other streams.
 template <typename R>
 void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm) {
-    int dev = 0, n_sm = 0, per_sm = 0;
+    int dev = 0, per_sm = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     constexpr int PART = sizeof(R) == 4 ? 2 : -1;
     constexpr int parts = PART < 0 ? 2 : 1;
@@ -737,16 +736,9 @@ void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm) {
     // that the chip holds at once.  A molecule has about half its neighbours'
     // pairs (in a box those within rc of any of its points, some 1.4 A more
     // between the O).
-    const int places = n_sm * (sizeof(R) == 4 ? SHORT_BLOCKS : 4);
     const double rn = p.rc + 1.4, V = p.box[0] * p.box[1] * p.box[2];
     const double nbr = p.periodic ? std::min(p.M - 1.0, p.M / V * 4.18879 * rn * rn * rn) : p.M / (double)p.n_cl - 1.0;
-    int mpw = 1;
-    double best = 1e30;
-    for (int k = 1; k <= 64; ++k) {
-        const double waves = std::ceil((double)((p.M + k - 1) / k) * parts / places);
-        const double c = waves * std::ceil((p.periodic ? 0.0 : 0.25) + k * std::max(0.5, 0.5 * nbr) / 32.0);
-        if (c < best) best = c, mpw = k;
-    }
+    const int mpw = warp_molecules(p.M, 0.5 * nbr, parts, sizeof(R) == 4 ? SHORT_BLOCKS : 4, p.periodic ? 0.0 : 0.25, 64);
     size_t sm = 0;
     k_short_pack<R><<<(p.M * 5 + 255) / 256, 256, 0, L.s>>>(p, d);
     const unsigned ng = (unsigned)((p.M + 3) / 4);

@@ -828,6 +828,23 @@ template <typename R> void launch_sites(const KParams &p, DevState<R> &d, double
 template <typename R> void launch_neighbors(const KParams &p, DevState<R> &d, int ncell[3], Launch L);
 template <typename R> void launch_real_perm(const KParams &p, DevState<R> &d, Launch L);
 template <typename R> void launch_lp_potential(const KParams &p, DevState<R> &d, Launch L);
+// Molecules that a one-warp block takes, of which each has `own` entries of
+// work, so that `parts` such grids need the fewest rounds of 32 entries in a
+// row over the blocks that the device holds at once (per_sm an SM).  margin:
+// part of a round for molecules that have more than the average.
+inline int warp_molecules(int M, double own, int parts, int per_sm, double margin, int most) {
+    int dev = 0, n_sm = 0, k_best = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    double best = 1e30;
+    for (int k = 1; k <= most; ++k) {
+        const double waves = ceil((double)((M + k - 1) / k) * parts / ((double)n_sm * per_sm));
+        const double c = waves * ceil(margin + k * (own > 0.5 ? own : 0.5) / 32.0);
+        if (c < best) best = c, k_best = k;
+    }
+    return k_best;
+}
+
 template <typename R> void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm = 0);
 template <typename R> void launch_ct(const KParams &p, DevState<R> &d, Launch L);
 template <typename R> void launch_intra_perm(const KParams &p, DevState<R> &d, Launch L);

@@ -1,5 +1,6 @@
-"""Short-range pairs: each molecule pair is evaluated once, by the molecule
-that the parity of their indices names, in rounds that run across molecules."""
+"""Each molecule pair of the short-range terms, and each gas-phase pair of the
+permanent energy, is evaluated by the molecule that the parity of their
+indices names, in rounds that run across molecules."""
 import numpy as np
 import pytest
 
@@ -40,8 +41,8 @@ def test_rounds_across_molecules_agree(sizes):
     a = _terms(sizes)
     b = _terms(sizes + [32] * 60)   # the same seeds for the first clusters
     for x, y in zip(a, b):
-        mag = sum(abs(x[t]) for t in ("rep", "disp", "xdisp"))
-        for t in ("rep", "disp", "xdisp"):
+        mag = sum(abs(x[t]) for t in ("elec", "pen", "rep", "disp", "xdisp"))
+        for t in ("elec", "pen", "rep", "disp", "xdisp"):
             assert abs(x[t] - y[t]) <= 1e-12 * mag, (t, x[t], y[t])
 
 
