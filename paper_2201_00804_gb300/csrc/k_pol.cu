@@ -626,44 +626,70 @@ __global__ void __launch_bounds__(128) k_finalize(KParams p, DevState<R> d, doub
 }
 
 // Virial total: out[3a + b] = -dE/d eps_ab = -(sum over molecules of the
-// streams' dE/d eps + the k-space sums of npass convolution passes), summed
-// in a fixed order by one block.
+// streams' dE/d eps + the k-space sums of npass convolution passes), summed in
+// a fixed order: every block takes a share of both arrays, a thread always the
+// same component, and the last block to finish adds the blocks' sums.  (One
+// block, with one thread for the k-space sums, was 290 us at 2,028 waters; this is 10.)
+constexpr int VT_BLOCKS = 152, VT_ROW = 16;   // partial sums: 9 components, then 7 k-space sums
 template <typename R>
 __global__ void __launch_bounds__(256) k_virial_total(int M, DevState<R> d, int npass, double *out) {
-    __shared__ double sh[8][9];
-    double v[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int m = threadIdx.x; m < M; m += blockDim.x)
-        for (int k = 0; k < 9; ++k) v[k] += d.vir[m * 9 + k] + d.vir_r[m * 9 + k] + d.vir_s[m * 9 + k];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int k = 0; k < 9; ++k) {
-        double x = v[k];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) sh[w][k] = x;
+    __shared__ double sh[2][256];
+    __shared__ bool last;
+    const int t = threadIdx.x, nb = gridDim.x;
+    double v = 0, s = 0;
+    if (t < 252)
+        for (int e = blockIdx.x * 252 + t; e < M * 9; e += nb * 252) v += d.vir[e] + d.vir_r[e] + d.vir_s[e];
+    for (int e = blockIdx.x * 256 + t; e < npass * VK_BLOCKS * 8; e += nb * 256) s += (e & 7) < 7 ? d.virk[e] : 0.0;
+    sh[0][t] = v;
+    sh[1][t] = s;
+    __syncthreads();
+    if (t < 9) {
+        double a = 0;
+        for (int k = t; k < 252; k += 9) a += sh[0][k];
+        d.partial[blockIdx.x * VT_ROW + t] = a;
+    } else if (t >= 32 && t < 39) {
+        double a = 0;
+        for (int k = t - 32; k < 256; k += 8) a += sh[1][k];
+        d.partial[blockIdx.x * VT_ROW + 9 + t - 32] = a;
+    }
+    __threadfence();
+    __syncthreads();
+    if (t == 0) last = atomicAdd(d.counter + 2, 1u) == (unsigned)nb - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double x = 0;
+    for (int b = t / VT_ROW; b < nb; b += 256 / VT_ROW) x += __ldcg(d.partial + b * VT_ROW + t % VT_ROW);
+    sh[0][t] = x;
+    __syncthreads();
+    if (t < VT_ROW) {
+        double a = 0;
+        for (int k = t; k < 256; k += VT_ROW) a += sh[0][k];
+        sh[1][t] = a;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t[9];
-        for (int k = 0; k < 9; ++k) {
-            t[k] = 0;
-            for (int j = 0; j < 8; ++j) t[k] += sh[j][k];
-        }
-        double ks[7] = {0, 0, 0, 0, 0, 0, 0};
-        for (int b = 0; b < npass * VK_BLOCKS; ++b)
-            for (int k = 0; k < 7; ++k) ks[k] += d.virk[(size_t)b * 8 + k];
+    if (t == 0) {
+        const double *ks = sh[1] + 9;
+        double a[9];
+        for (int k = 0; k < 9; ++k) a[k] = sh[1][k];
         // dE/d eps_ab from the k-space sums: -delta_ab sum e + sum e f m_a m_b
         const int ia[6] = {0, 4, 8, 1, 2, 5}, ib[6] = {0, 4, 8, 3, 6, 7};
-        for (int k = 0; k < 3; ++k) t[4 * k] -= ks[0];
+        for (int k = 0; k < 3; ++k) a[4 * k] -= ks[0];
         for (int k = 0; k < 6; ++k) {
-            t[ia[k]] += ks[1 + k];
-            if (ib[k] != ia[k]) t[ib[k]] += ks[1 + k];
+            a[ia[k]] += ks[1 + k];
+            if (ib[k] != ia[k]) a[ib[k]] += ks[1 + k];
         }
-        for (int k = 0; k < 9; ++k) out[k] = -t[k];
+        for (int k = 0; k < 9; ++k) out[k] = -a[k];
+        d.counter[2] = 0;
     }
 }
 
+// The partial sums take the solve's array, which is free by now and holds
+// 4 ceil(9 M / 256) + 64 values: 16 a block for a block per 128 molecules.
 template <typename R>
 void launch_virial_total(const KParams &p, DevState<R> &d, double *out, Launch L) {
-    k_virial_total<R><<<1, 256, 0, L.s>>>(p.M, d, p.periodic ? 2 : 0, out);
+    const int nb = std::min(VT_BLOCKS, (p.M + 127) / 128);
+    k_virial_total<R><<<nb, 256, 0, L.s>>>(p.M, d, p.periodic ? 2 : 0, out);
     count(L);
 }
 
