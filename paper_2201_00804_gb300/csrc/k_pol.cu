@@ -331,6 +331,103 @@ __global__ void __launch_bounds__(PB) k_pcg_step(KParams p, DevState<R> d, cudaG
     zero_grid(p, d, tid, nth);
 }
 
+// The same for one system of at most one element a thread: what a thread owns
+// stays in registers from the product to the next direction (z and T p are
+// never stored, mu and r are read before the first wait), and the step lengths
+// are each one thread's division.  A step is a chain of latencies, two grid
+// barriers among them; FP64 quotients and roots in every warp were some 4 us of
+// it.  2,028 waters 16.0 -> 13.1 us, 4,096 waters 18.7 -> 13.5.  (With four elements a
+// thread, 32,000 waters, 29.1 -> 21.2 alone, but the evaluation stays as long:
+// there the other streams' work fills the waits.)
+template <typename R>
+__global__ void __launch_bounds__(PB, 2) k_pcg_step_regs(KParams p, DevState<R> d, cudaGraphConditionalHandle loop,
+                                                         int maxit) {
+    namespace cg = cooperative_groups;
+    cg::grid_group grid = cg::this_grid();
+    __shared__ double sh[32];
+    __shared__ double s_v[2];
+    if (d.flags[1]) {
+        if (maxit > 0 && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(loop, 0u);
+        return;
+    }
+    const int n = p.M * 9, k = blockIdx.x * PB + threadIdx.x, nb = gridDim.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double rz_old = d.scal[S_RZ], tol = d.scal[S_TOL];
+    double pv = 0, ap = 0, mu = 0, r = 0, pap = 0;
+    if (k < n) {
+        pv = d.pv[k];
+        mu = d.mu[k];
+        r = d.res[k];
+        ap = pv * apol_inv(p, k) - (d.efp[k] + d.efp_r[k]);
+        pap = pv * ap;
+    }
+    pap = block_sum(pap, sh);
+    if (threadIdx.x == 0) d.partial[blockIdx.x] = pap;
+    grid.sync();
+    if (w == 0) {
+        double v = 0;
+        for (int b = lane; b < nb; b += 32) v += __ldcg(d.partial + b);
+        v = warp_sum(v);
+        if (lane == 0) {
+            s_v[0] = v;
+            s_v[1] = rz_old / v;
+        }
+    }
+    __syncthreads();
+    const double tpap = s_v[0], al = s_v[1];
+    double rz = 0, rr = 0;
+    if (k < n) {
+        d.mu[k] = mu + al * pv;
+        r -= al * ap;
+        d.res[k] = r;
+        const double z = apol(p, k) * r;
+        rz = r * z;
+        rr = z * z;
+        r = z;
+    }
+    double brz, brr;
+    block_sum2(rz, rr, sh, brz, brr);
+    if (threadIdx.x == 0) {
+        d.partial[nb + 2 * blockIdx.x] = brz;
+        d.partial[nb + 2 * blockIdx.x + 1] = brr;
+    }
+    grid.sync();
+    __shared__ double s_t[2];
+    if (w < 2) {   // warp 0: r.z and the direction's step, warp 1: the residual
+        double v = 0;
+        for (int b = lane; b < nb; b += 32) v += __ldcg(d.partial + nb + 2 * b + w);
+        v = warp_sum(v);
+        if (lane == 0) {
+            s_t[w] = v;
+            s_v[w] = w == 0 ? v / rz_old : sqrt(v / (p.M * 3)) * 4.80321;
+        }
+    }
+    __syncthreads();
+    const double beta = s_v[0], res = s_v[1];
+    const bool done = res < tol;
+    if (k == 0) {
+        d.scal[S_PAP] = tpap;
+        d.scal[S_ALPHA] = al;
+        d.scal[S_BETA] = beta;
+        d.scal[S_RZ] = s_t[0];
+        d.scal[S_RES] = res;
+        d.scal[S_IT] += 1.0;
+        if (done) {
+            d.scal[S_DONE] = 1.0;
+            d.flags[1] = 1;
+        }
+        if (maxit > 0) cudaGraphSetConditional(loop, (!done && d.scal[S_IT] < (double)maxit) ? 1u : 0u);
+    }
+    if (done) return;   // uniform: every block computed the same residual
+    if (k < n) {
+        const double pk = r + beta * pv;
+        d.pv[k] = pk;
+        d.vecR[k] = R(pk);
+        d.efp[k] = 0.0;
+        d.efp_r[k] = 0.0;
+    }
+    zero_grid(p, d, k, (size_t)nb * PB);
+}
+
 static inline unsigned nblk(int n) { return (unsigned)((n + PB - 1) / PB); }
 
 // after the solve: record a solve that stopped at the iteration limit
@@ -357,22 +454,26 @@ void launch_pcg_first(const KParams &p, DevState<R> &d, Launch L) {
     k_pcg_first<R><<<nblk(p.M * 9), PB, 0, L.s>>>(p, d);
     count(L);
 }
-// Cooperative launch of the PCG step: a grid-stride kernel with as many
-// blocks as can be resident at once (at most one per 256 vector entries).
+// Cooperative launch of the PCG step: at most two blocks per SM (the grid must
+// be co-resident while the short-range kernels occupy part of every SM on
+// their own stream) and one per 256 vector entries.
 template <typename R>
 void launch_pcg_step(const KParams &p, DevState<R> &d, Launch L, cudaGraphConditionalHandle loop, int maxit) {
-    static int per_sm[2] = {0, 0}, n_sm = 0;
-    int &ps = per_sm[sizeof(R) == 8];
-    if (ps == 0) {
+    static int per_sm[2][2] = {}, n_sm = 0;
+    decltype(&k_pcg_step<R>) ks[2] = {k_pcg_step<R>, k_pcg_step_regs<R>};
+    int *ps = per_sm[sizeof(R) == 8];
+    if (ps[1] == 0) {
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_pcg_step<R>, PB, 0);
-        if (ps < 1) ps = 1;
+        for (int v = 0; v < 2; ++v) {
+            int b = 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, ks[v], PB, 0);
+            ps[v] = std::max(1, std::min(b, 2));
+        }
     }
-    // at most two blocks per SM: the grid must be co-resident while the
-    // short-range kernels occupy part of every SM on their own stream
-    const unsigned grid = (unsigned)std::min<long long>(nblk(p.M * 9), (long long)std::min(ps, 2) * n_sm);
+    const int n = p.M * 9, v = p.n_cl == 1 && n <= ps[1] * n_sm * PB;
+    const unsigned grid = (unsigned)std::min<long long>(nblk(n), (long long)ps[v] * n_sm);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(PB);
@@ -382,7 +483,7 @@ void launch_pcg_step(const KParams &p, DevState<R> &d, Launch L, cudaGraphCondit
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_pcg_step<R>, p, d, loop, maxit);
+    cudaLaunchKernelEx(&cfg, ks[v], p, d, loop, maxit);
     count(L);
 }
 
