@@ -554,21 +554,29 @@ void launch_real_perm(const KParams &p, DevState<R> &d, Launch L) {
 }
 
 // Potential of the permanent multipoles and its gradient at the lone pairs
-// (ATOMS = false) or, for the original charge transfer, at O, H1 and H2: one
-// point per warp, the five source sites sharing one queue.
+// (ATOMS = false) or, for the original charge transfer, at O, H1 and H2: the
+// five source sites share one queue.  FP32: a warp takes all of a molecule's
+// points, which share the list walk, the queue and the source loads (32,000
+// waters 270 us, a warp per point 376; 4096 clusters of 17 waters 109 and 155);
+// FP64, bound by its pipe: a warp per point, which spreads the work.
 constexpr int QCAP_P = 192;   // >= 31 carried + 5 sites x 32 new entries
 template <typename R, bool PER, bool ATOMS>
 __global__ void __launch_bounds__(128) k_potential(KParams p, DevState<R> d) {
-    constexpr int NPT = ATOMS ? 3 : 2;   // points a molecule
+    constexpr int NPT = ATOMS ? 3 : 2;                     // points a molecule
+    constexpr int PW = sizeof(R) == 4 ? NPT : 1;           // points a warp
     __shared__ PairQueue<R, QCAP_P> qs[4];
     const int wq = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int a = blockIdx.x * 4 + wq, i = a / NPT;
+    const int a = (blockIdx.x * 4 + wq) * PW, i = a / NPT;   // first point, molecule
     if (i >= p.M) return;
     PairQueue<R, QCAP_P> &q = qs[wq];
-    const V3<R> ot = my_pt(d, i, (ATOMS ? 0 : NS) + a % NPT);
+    V3<R> ot[PW], gr[PW];
+    Acc<R> V[PW];
+#pragma unroll
+    for (int u = 0; u < PW; ++u) {
+        ot[u] = my_pt(d, i, (ATOMS ? 0 : NS) + a % NPT + u);
+        gr[u] = mk(R(0), R(0), R(0));
+    }
     const R rc2 = sc<R>(p).rc2, alpha = sc<R>(p).alpha;
-    Acc<R> V;
-    V3<R> gr = mk(R(0), R(0), R(0));
     int h = 0, t = 0;
     const int nn = d.nnbr[i];
     for (int base = 0;; base += 32) {
@@ -584,12 +592,18 @@ __global__ void __launch_bounds__(128) k_potential(KParams p, DevState<R> d) {
             const R *offj = d.off + j * NP * 3;
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
-                const V3<R> os = mk(__ldg(offj + s * 3), __ldg(offj + s * 3 + 1), __ldg(offj + s * 3 + 2));
-                // periodic: the source position; gas phase: the displacement
-                // formed as (target - source offset) - D, queued itself
-                rs[s] = PER ? dO + os : (ot - os) - dO;
-                const V3<R> x = ot - rs[s];
-                if (!PER || dot(x, x) < rc2) bits |= 1u << s;
+                // queued: the source position in a box, the displacement of the molecules in the gas phase
+                rs[s] = dO;
+                if (!PER) {
+                    bits |= 1u << s;
+                    continue;
+                }
+                rs[s] = dO + mk(__ldg(offj + s * 3), __ldg(offj + s * 3 + 1), __ldg(offj + s * 3 + 2));
+#pragma unroll
+                for (int u = 0; u < PW; ++u) {
+                    const V3<R> x = ot[u] - rs[s];
+                    if (dot(x, x) < rc2) bits |= 1u << s;
+                }
             }
         }
         int n;
@@ -602,13 +616,22 @@ __global__ void __launch_bounds__(128) k_potential(KParams p, DevState<R> d) {
         while (t - h >= 32 || (flush && t > h)) {
             if (lane < t - h) {
                 const int e = (h + lane) % QCAP_P, js = q.js[e];
-                const V3<R> x = PER ? ot - q.at(e) : q.at(e);
-                const Source<R> src(scaled(load_mp_g(d.gmp + ((js >> 3) * NS + (js & 7)) * GMP), R(1.0 / 3.0)), x);
-                const R r2 = dot(x, x), rinv = rsqrt_(r2), r2i = rinv * rinv;
-                R B[4];
-                kernel_B<R, PER, 3>(r2 * rinv, rinv, r2i, alpha, B);
-                V.add(src.q * B[0] + src.s * B[1] + src.w * B[2]);
-                gr = gr + src.grad(x, B[1], B[2], B[3]);
+                const Mp<R> ms = scaled(load_mp_g(d.gmp + ((js >> 3) * NS + (js & 7)) * GMP), R(1.0 / 3.0));
+                V3<R> os = mk(R(0), R(0), R(0));
+                if (!PER) os = my_pt(d, js >> 3, js & 7);
+#pragma unroll
+                for (int u = 0; u < PW; ++u) {
+                    // gas phase: formed as (target - source offset) - D
+                    const V3<R> x = PER ? ot[u] - q.at(e) : (ot[u] - os) - q.at(e);
+                    const R r2 = dot(x, x);
+                    if (PER && PW > 1 && !(r2 < rc2)) continue;   // queued for another point
+                    const Source<R> src(ms, x);
+                    const R rinv = rsqrt_(r2), r2i = rinv * rinv;
+                    R B[4];
+                    kernel_B<R, PER, 3>(r2 * rinv, rinv, r2i, alpha, B);
+                    V[u].add(src.q * B[0] + src.s * B[1] + src.w * B[2]);
+                    gr[u] = gr[u] + src.grad(x, B[1], B[2], B[3]);
+                }
             }
             h += min(32, t - h);
         }
@@ -616,16 +639,22 @@ __global__ void __launch_bounds__(128) k_potential(KParams p, DevState<R> d) {
         if (flush) break;
     }
     const double ke = p.ke;
-    const double v = warp_sum_acc(V);
-    const R vals[3] = {gr.x, gr.y, gr.z};
-    const R g = warp_transpose_sum<R, 3>(vals, reinterpret_cast<R *>(&q), lane);
-    if (lane < 3) (ATOMS ? d.dva : d.dvlp)[a * 3 + lane] += ke * double(g);
-    if (lane == 0) (ATOMS ? d.va : d.vlp)[a] += ke * v;
+    R vals[3 * PW];
+#pragma unroll
+    for (int u = 0; u < PW; ++u) vals[3 * u] = gr[u].x, vals[3 * u + 1] = gr[u].y, vals[3 * u + 2] = gr[u].z;
+    const R g = warp_transpose_sum<R, 3 * PW>(vals, reinterpret_cast<R *>(&q), lane);
+    if (lane < 3 * PW) (ATOMS ? d.dva : d.dvlp)[a * 3 + lane] += ke * double(g);
+#pragma unroll
+    for (int u = 0; u < PW; ++u) {
+        const double v = warp_sum_acc(V[u]);
+        if (lane == 0) (ATOMS ? d.va : d.vlp)[a + u] += ke * v;
+    }
 }
 
 template <typename R, bool ATOMS>
 void launch_potential(const KParams &p, DevState<R> &d, Launch L) {
-    const unsigned nb = (unsigned)((p.M * (ATOMS ? 3 : 2) + 3) / 4);
+    const int warps = p.M * (sizeof(R) == 4 ? 1 : (ATOMS ? 3 : 2));
+    const unsigned nb = (unsigned)((warps + 3) / 4);
     if (p.periodic) k_potential<R, true, ATOMS><<<nb, 128, 0, L.s>>>(p, d);
     else k_potential<R, false, ATOMS><<<nb, 128, 0, L.s>>>(p, d);
     count(L);
