@@ -602,13 +602,15 @@ sibfa_status fft(sibfa_ctx *ctx, DevState<R> &d, bool forward, int ngrid) {
 
 // The grids' convolution with the influence function on s2 (permanent and
 // force passes): in one kernel for the small systems whose solve runs in one
-// too, where the chain of transforms is on the critical path (216 waters: 66 ->
-// 53 and 71 -> 58 us a pass, FP64 198 -> 162 and 247 -> 216); the library's
+// too, where the chain of transforms is on the critical path (216 waters: force
+// pass 71 -> 58 us, FP64 198 -> 162 and 247 -> 216 us a pass); the library's
 // transforms otherwise (32,000 waters, products included: 8454 us a call
-// against 8597).
+// against 8597), and for the FP32 permanent grid: its energy nearly cancels
+// against the self terms, and the one kernel's rounded twiddles shift it by
+// 1.3e-7 of the electrostatic energy (53 us a pass against 66).
 template <typename R>
 sibfa_status convolve(sibfa_ctx *ctx, DevState<R> &d, int ngrid, Launch L2) {
-    if (ctx->conv.ncta > 0) {
+    if (ctx->conv.ncta > 0 && (sizeof(R) == 8 || ngrid == 2)) {
         CK(launch_grid_conv(ctx->kp, d, ctx->conv, ngrid, L2));
         return SIBFA_OK;
     }
