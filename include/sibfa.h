@@ -253,7 +253,8 @@ sibfa_status sibfa_cluster_terms(sibfa_ctx *ctx, sibfa_energy_terms *terms);
 uint64_t sibfa_kernel_launches(const sibfa_ctx *ctx);
 
 /* Launch shape of the short-range kernels chosen by the context's tuning:
- * *blocks_per_sm = resident blocks per SM (0 = uncapped), *done = 1 once the
+ * *blocks_per_sm = resident blocks per SM (0 = uncapped; on the mixed path a
+ * block stands for four warps), *done = 1 once the
  * tuning has fixed it (0 while candidates are still being timed).  Either
  * pointer may be NULL.  Returns SIBFA_E_INVALID for a NULL context. */
 sibfa_status sibfa_tuned_shape(const sibfa_ctx *ctx, int *blocks_per_sm, int *done);

@@ -3,7 +3,7 @@
 // Every kernel walks the neighbours of one molecule i and accumulates only
 // i's quantities (energy halves, gradients of i's points, multipole
 // sensitivities of i's sites), so no two threads write the same output and
-// no atomics are needed; the neighbour list is full, each molecule pair is
+// no atomics are needed (k_perm_gas: two warps add to a target); the neighbour list is full, each molecule pair is
 // visited from both sides.  Pair arithmetic runs in R (float in the mixed
 // path, double in the FP64 path); per-lane partial sums are reduced across
 // the warp in double.
@@ -38,7 +38,7 @@ __device__ __forceinline__ void symacc(Sym<R> &a, const Sym<R> &b) {
 // The target kernels below run one target site per block of one warp.  They
 // are bound by issue and by the latency of each round's source loads, so what
 // counts is warps per SM: blocks of one warp take any register count that
-// divides the file (112 registers, 18 warps, against 15 in blocks of five),
+// divides the file (96 registers, 21 warps, against 15 in blocks of five),
 // and a molecule's heavy targets (atoms) do not hold up its light ones.
 // ---------------------------------------------------------------------------
 constexpr int QCAP_A = 128;   // >= 31 carried + 3 atom sites x 32 new entries
@@ -338,9 +338,9 @@ int gas_mpw(const KParams &p) {
                           sizeof(R) == 4 ? 32 : 4);
 }
 
-// Boxes.  Blocks per SM, FP32: 18 (112 registers; 32,000 waters: 1728 us,
-// 1909 at 16, 1735 at 20, where registers spill, 1926 with the five sites in
-// one block); FP64 8 (216 waters: 274 us against 416 in one block).
+// Boxes.  Blocks per SM, FP32: at least 18 (96 registers, 21 blocks; 32,000 waters
+// 1630 us; at 112 registers and 18 blocks 1728, with the five sites in one
+// block 1926); FP64 8 (216 waters: 274 us against 416 in one block).
 template <typename R, bool VIR>
 __global__ void __launch_bounds__(VIR ? 32 * NS : 32,
                                   VIR ? (sizeof(R) == 4 ? 3 : 2) : (sizeof(R) == 4 ? 18 : 8))

@@ -722,9 +722,9 @@ __global__ void __launch_bounds__(128) k_short_gather(KParams p, DevState<R> d, 
 
 }  // namespace
 
-// max_per_sm > 0 caps the warps resident per SM at four times that by reserving
-// unused dynamic shared memory, which leaves registers on every SM for the
-// kernels of the other streams.
+// max_per_sm > 0 caps the resident blocks per SM (FP32: warps, at four times
+// that) by reserving unused dynamic shared memory, which leaves registers on
+// every SM for the kernels of the other streams.
 template <typename R>
 void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm) {
     int dev = 0, per_sm = 0;
@@ -744,11 +744,11 @@ void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm) {
     const unsigned ng = (unsigned)((p.M + 3) / 4);
     auto run = [&](auto per, auto vir) {
         auto k = k_short<R, decltype(per)::value, decltype(vir)::value, PART>;
-        if (max_per_sm > 0 && !p.vir) {
+        const int cap = sizeof(R) == 4 ? 4 * max_per_sm : max_per_sm;
+        if (cap > 0 && cap < SHORT_BLOCKS && !p.vir) {   // (registers allow no more than SHORT_BLOCKS)
             cudaFuncAttributes fa;
             cudaFuncGetAttributes(&fa, k);
             // one byte more per block than another block would leave room for
-            const int cap = sizeof(R) == 4 ? 4 * max_per_sm : max_per_sm;
             const long long need = per_sm / (cap + 1) + 1 - (long long)fa.sharedSizeBytes - 1024;
             if (need > 0) {
                 sm = (size_t)need;
