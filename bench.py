@@ -787,13 +787,14 @@ def main():
     else:
         units = count_units_clusters(o["cluster_start"], M)
     kfl = kernel_flops(units)
-    kernels = {"real_perm": ("k_real_perm<float, %d, 0, 0, 5, 0>" % int(args.workload != "clusters4096"),
+    periodic = args.workload != "clusters4096"
+    kernels = {"real_perm": ("k_real_perm<float, 0>" if periodic else "k_perm_gas<float, 0>",
                              "site targets: multipole + penetration energy, gradient, torque sensitivities, "
                              "Thole field; 1 launch per step"),
-               "short": ("k_short<float, %d, 0, 0|1>" % int(args.workload != "clusters4096"),
-                         "repulsion (part 0) and dispersion + exchange-dispersion (part 1); 2 launches per step, "
-                         "timed together"),
-               "ct": ("k_ct<float, %d, 0>" % int(args.workload != "clusters4096"),
+               "short": ("k_short<float, %d, 0, 2>" % int(periodic),
+                         "repulsion, dispersion + exchange-dispersion, each molecule pair once; timed with the "
+                         "packing and k_short_gather launches of the step"),
+               "ct": ("k_ct<float, %d, 0>" % int(periodic),
                       "reduced charge transfer; 1 launch per step")}
     lines = {}
     for key, (kname, what) in kernels.items():
