@@ -1214,6 +1214,7 @@ sibfa_status create_impl(sibfa_ctx *ctx, const sibfa_topology *topo) {
         CK(cudaMemcpyAsync(d.cl_of, of.data(), M * sizeof(int), cudaMemcpyHostToDevice, ctx->s));
     }
     CK(cudaStreamSynchronize(ctx->s));
+    if (ctx->cluster_max > 0) CK(cluster_init());
     // the solve in one kernel: one system whose grid axes factor into small
     // primes (cluster batches stop on each cluster's residual; the host loop
     // is for profilers)

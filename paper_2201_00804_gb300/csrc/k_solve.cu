@@ -1200,14 +1200,15 @@ cudaError_t launch_pcg_loop(const KParams &p, DevState<R> &d, const LoopPlan &lp
                       : cudaLaunchKernelEx(&cfg, k_pcg_loop<R, false>, p, d, lp, g, warm, push);
 }
 
+// The limit belongs to the process: always the largest cluster's, so that no
+// context lowers it between another thread's setting and its launch.
+cudaError_t cluster_init() {
+    return cudaFuncSetAttribute(k_pcg_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem(CLUSTER_MAX));
+}
+
 cudaError_t launch_pcg_cluster(const KParams &p, DevState<float> &d, int nmax, int maxit, const MuGuess &g, int warm,
                                double *push, Launch L) {
-    const size_t sm = cluster_smem(nmax);
-    if (sm > 40000) {
-        const cudaError_t e = cudaFuncSetAttribute(k_pcg_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
-    k_pcg_cluster<<<p.n_cl, CT, sm, L.s>>>(p, d, maxit, g, warm, push);
+    k_pcg_cluster<<<p.n_cl, CT, cluster_smem(nmax), L.s>>>(p, d, maxit, g, warm, push);
     count(L);
     return cudaGetLastError();
 }

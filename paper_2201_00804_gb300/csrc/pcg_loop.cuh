@@ -61,6 +61,8 @@ cudaError_t launch_pcg_loop(const KParams &p, DevState<R> &d, const LoopPlan &lp
 // Largest cluster the per-cluster solve takes (waters): its displacements,
 // n (n - 1) of them, stay in shared memory (48 KB at 64 waters).
 constexpr int CLUSTER_MAX = 64;
+// Admits the largest cluster's shared memory; once per context, at creation.
+cudaError_t cluster_init();
 // Every cluster of a gas-phase batch (mixed path) on its own, one block each; nmax: the largest.
 cudaError_t launch_pcg_cluster(const KParams &p, DevState<float> &d, int nmax, int maxit, const MuGuess &g, int warm,
                                double *push, Launch L);

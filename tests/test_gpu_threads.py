@@ -1,0 +1,62 @@
+"""Contexts on several host threads at once, as the server's slots are: a
+launch in one thread must not depend on what another thread sets."""
+import threading
+
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2201_00804_gb300 import build
+    build.build()
+
+
+def _together(jobs):
+    """Runs the callables on a thread each and raises the first error."""
+    errors = []
+
+    def run(f):
+        try:
+            f()
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=run, args=(f,)) for f in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    if errors:
+        raise errors[0]
+
+
+def test_clusters_of_several_sizes_on_several_threads():
+    """Single clusters of 44 and 64 waters (mixed path), each in steps of its
+    own thread.  The dipole history keeps every step a launch of its own."""
+    import torch
+    import paper_2201_00804_gb300 as pkg
+
+    def job(n):
+        def steps():
+            s = synth.make_cluster(n, seed=n)
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                pos = torch.tensor(s.pos.reshape(-1), dtype=torch.float64, device="cuda")
+                m = torch.tensor(s.masses().reshape(-1), dtype=torch.float64, device="cuda")
+                ctx = pkg.sibfa_create(synth.PARAMS, s.mp_local, periodic=False, pcg_tol_D=1e-4,
+                                       precision=pkg.PREC_MIXED, warm_start=2)
+                try:
+                    for _ in range(20):
+                        pkg.sibfa_md_steps(ctx, pos.clone(), torch.zeros_like(pos), m, 0.01, 100)
+                finally:
+                    pkg.sibfa_destroy(ctx)
+        return steps
+
+    _together([job(n) for n in (44, 64)])
