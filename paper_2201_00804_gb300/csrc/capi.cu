@@ -1215,6 +1215,7 @@ sibfa_status create_impl(sibfa_ctx *ctx, const sibfa_topology *topo) {
     }
     CK(cudaStreamSynchronize(ctx->s));
     if (ctx->cluster_max > 0) CK(cluster_init());
+    CK(short_init<R>(ctx->kp));
     // the solve in one kernel: one system whose grid axes factor into small
     // primes (cluster batches stop on each cluster's residual; the host loop
     // is for profilers)

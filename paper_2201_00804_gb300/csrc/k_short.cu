@@ -722,6 +722,25 @@ __global__ void __launch_bounds__(128) k_short_gather(KParams p, DevState<R> d, 
 
 }  // namespace
 
+template <typename R, bool PER>
+static cudaError_t short_admit() {
+    constexpr int PART = sizeof(R) == 4 ? 2 : -1;
+    const auto k = k_short<R, PER, false, PART>;
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+    return e;
+}
+// Admits any reservation of launch_short, once per context, at creation: the
+// limit belongs to the process, so a launch that set its own could be refused
+// when another thread's context lowered it in between.
+template <typename R>
+cudaError_t short_init(const KParams &p) { return p.periodic ? short_admit<R, true>() : short_admit<R, false>(); }
+
 // max_per_sm > 0 caps the resident blocks per SM (FP32: warps, at four times
 // that) by reserving unused dynamic shared memory, which leaves registers on
 // every SM for the kernels of the other streams.
@@ -750,10 +769,7 @@ void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm) {
             cudaFuncGetAttributes(&fa, k);
             // one byte more per block than another block would leave room for
             const long long need = per_sm / (cap + 1) + 1 - (long long)fa.sharedSizeBytes - 1024;
-            if (need > 0) {
-                sm = (size_t)need;
-                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            }
+            if (need > 0) sm = (size_t)need;   // (short_init admits it)
         }
         k<<<dim3((unsigned)((p.M + mpw - 1) / mpw), parts), 32, sm, L.s>>>(p, d, mpw);
         k_short_gather<R, decltype(per)::value, decltype(vir)::value><<<ng, 128, 0, L.s>>>(p, d, parts);
@@ -763,6 +779,8 @@ void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm) {
     count(L, 3);
 }
 
+template cudaError_t short_init<float>(const KParams &);
+template cudaError_t short_init<double>(const KParams &);
 template void launch_short<float>(const KParams &, DevState<float> &, Launch, int);
 template void launch_short<double>(const KParams &, DevState<double> &, Launch, int);
 

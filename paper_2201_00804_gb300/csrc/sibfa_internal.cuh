@@ -845,6 +845,7 @@ inline int warp_molecules(int M, double own, int parts, int per_sm, double margi
     return k_best;
 }
 
+template <typename R> cudaError_t short_init(const KParams &p);
 template <typename R> void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm = 0);
 template <typename R> void launch_ct(const KParams &p, DevState<R> &d, Launch L);
 template <typename R> void launch_intra_perm(const KParams &p, DevState<R> &d, Launch L);

@@ -60,3 +60,26 @@ def test_clusters_of_several_sizes_on_several_threads():
         return steps
 
     _together([job(n) for n in (44, 64)])
+
+
+def test_short_range_caps_on_several_threads():
+    """FP64 contexts whose schedule tuning is under way: each tries caps of 3,
+    0 and 2 blocks per SM, which reserve different amounts of shared memory."""
+    import numpy as np
+    import paper_2201_00804_gb300 as pkg
+
+    def job(k):
+        def calls():
+            s = synth.make_cluster(2, seed=70 + k)
+            pos = np.ascontiguousarray(s.pos.reshape(-1))
+            for _ in range(120):
+                ctx = pkg.sibfa_create(synth.PARAMS, s.mp_local, periodic=False, pcg_tol_D=1e-4,
+                                       precision=pkg.PREC_FP64, warm_start=False)
+                try:
+                    for _ in range(12):
+                        pkg.sibfa_energy_forces(ctx, pos)
+                finally:
+                    pkg.sibfa_destroy(ctx)
+        return calls
+
+    _together([job(k) for k in range(6)])
