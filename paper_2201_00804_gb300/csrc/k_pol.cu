@@ -459,21 +459,24 @@ void launch_pcg_first(const KParams &p, DevState<R> &d, Launch L) {
 // their own stream) and one per 256 vector entries.
 template <typename R>
 void launch_pcg_step(const KParams &p, DevState<R> &d, Launch L, cudaGraphConditionalHandle loop, int maxit) {
-    static int per_sm[2][2] = {}, n_sm = 0;
     decltype(&k_pcg_step<R>) ks[2] = {k_pcg_step<R>, k_pcg_step_regs<R>};
-    int *ps = per_sm[sizeof(R) == 8];
-    if (ps[1] == 0) {
+    struct Resident {
+        int n_sm = 0, per_sm[2];
+    };
+    static const Resident res = [&] {   // on first use, whichever thread's it is
+        Resident q;
         int dev = 0;
         cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&q.n_sm, cudaDevAttrMultiProcessorCount, dev);
         for (int v = 0; v < 2; ++v) {
             int b = 0;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, ks[v], PB, 0);
-            ps[v] = std::max(1, std::min(b, 2));
+            q.per_sm[v] = std::max(1, std::min(b, 2));
         }
-    }
-    const int n = p.M * 9, v = p.n_cl == 1 && n <= ps[1] * n_sm * PB;
-    const unsigned grid = (unsigned)std::min<long long>(nblk(n), (long long)ps[v] * n_sm);
+        return q;
+    }();
+    const int n = p.M * 9, v = p.n_cl == 1 && n <= res.per_sm[1] * res.n_sm * PB;
+    const unsigned grid = (unsigned)std::min<long long>(nblk(n), (long long)res.per_sm[v] * res.n_sm);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(PB);

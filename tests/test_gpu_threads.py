@@ -83,3 +83,40 @@ def test_short_range_caps_on_several_threads():
         return calls
 
     _together([job(k) for k in range(6)])
+
+
+FIRST_SOLVES = """
+import threading
+import numpy as np
+import synth
+import paper_2201_00804_gb300 as pkg
+
+s = synth.make_cluster(30, seed=80)
+pos = np.ascontiguousarray(s.pos.reshape(-1))
+ctx = [pkg.sibfa_create(synth.PARAMS, s.mp_local, periodic=False, pcg_tol_D=1e-8, precision=pkg.PREC_FP64,
+                        warm_start=False) for _ in range(8)]
+start, pol = threading.Barrier(8), []
+
+def first(c):
+    start.wait()
+    pol.append(pkg.sibfa_energy_forces(c, pos)["pol"])
+
+threads = [threading.Thread(target=first, args=(c,)) for c in ctx]
+for t in threads:
+    t.start()
+for t in threads:
+    t.join()
+assert len(pol) == 8 and max(pol) - min(pol) <= 1e-9 * abs(pol[0]), pol
+"""
+
+
+def test_first_solves_of_a_process_on_several_threads():
+    """The first solves by separate kernels of a process, at the same time:
+    each sees the launch shape that the first of them lays down."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FIRST_SOLVES], cwd=root, env=dict(os.environ, SIBFA_PCG_HOST_LOOP="1"),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
