@@ -928,7 +928,7 @@ def main():
                 "temperature_end_K": 2.0 * kinetic(vel, masses.repeat_interleave(3)) / ((vel.numel() - 3) * KB_KCAL)},
         "tuned": {"short_blocks_per_sm": tb, "short_joined_before_solve": tjoin, "fixed": tdone,
                   "candidates_ms": {f"{c}{'+join' if j else ''}": round(t, 4)
-                                    for (c, j), t in zip(((3, 0), (0, 0), (2, 0), (0, 1), (3, 1)), tms)}},
+                                    for (c, j), t in zip(((3, 0), (0, 0), (2, 0), (0, 1), (3, 1)), tms) if t > 0}},
         "npt": npt,
     }
     print(json.dumps(line), flush=True)

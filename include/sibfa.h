@@ -253,15 +253,16 @@ sibfa_status sibfa_cluster_terms(sibfa_ctx *ctx, sibfa_energy_terms *terms);
 uint64_t sibfa_kernel_launches(const sibfa_ctx *ctx);
 
 /* Launch shape of the short-range kernels chosen by the context's tuning:
- * *blocks_per_sm = resident blocks per SM (0 = uncapped; on the mixed path a
- * block stands for four warps), *done = 1 once the
+ * *blocks_per_sm = resident blocks per SM (0 = uncapped, as always on the
+ * mixed path), *done = 1 once the
  * tuning has fixed it (0 while candidates are still being timed).  Either
  * pointer may be NULL.  Returns SIBFA_E_INVALID for a NULL context. */
 sibfa_status sibfa_tuned_shape(const sibfa_ctx *ctx, int *blocks_per_sm, int *done);
 
 /* The whole short-range schedule chosen by the tuning.  The candidates, in
  * order: (blocks per SM, joined before the solve) = (3, no), (0, no),
- * (2, no), (0, yes), (3, yes); "joined before the solve" means the
+ * (2, no), (0, yes), (3, yes), on the mixed path only the two without a
+ * cap; "joined before the solve" means the
  * short-range kernels finish before the polarization solve starts (the
  * solve's latency-bound kernels then have the SMs to themselves), otherwise
  * they run beside it until the chain rule.  *blocks_per_sm, *join_before_solve

@@ -34,18 +34,19 @@ struct sibfa_ctx {
     cudaStream_t s3 = nullptr;
     cudaEvent_t ev_fork3 = nullptr, ev_join3 = nullptr;
     bool short_pending = false;
-    // Autotuner of the short-range schedule: resident blocks per SM (0 =
-    // uncapped) and whether the short-range stream is joined before the
+    // Autotuner of the short-range schedule: resident blocks per SM (FP64 path;
+    // 0 = uncapped) and whether the short-range stream is joined before the
     // polarization solve (the solve then has the SMs to itself) or only
     // before the chain rule.  The first evaluations outside sibfa_minimize
     // after two warm-up ones
     // each run one candidate and are timed whole on the main stream (two per
-    // candidate, the faster kept); then the fastest candidate is fixed.  The
-    // choice changes only the scheduling, never the arithmetic.
+    // candidate in FP64, four in the mixed path, the fastest kept); then the
+    // fastest candidate is fixed.  The choice changes only the scheduling, never
+    // the arithmetic.
     struct ShortTuner {
         bool on = true;
         int seen = 0;            // evaluations with forces seen
-        int cand = 0;            // candidate being timed
+        int cand = 0;            // candidate being timed (place in the precision's list)
         int reps = 0;
         int choice = -1;         // fixed candidate, -1 while tuning
         float tmin[5] = {1e30f, 1e30f, 1e30f, 1e30f, 1e30f};
@@ -501,22 +502,33 @@ sibfa_status join_ct(sibfa_ctx *ctx) {
 }
 
 // Short-range schedule candidates: resident blocks per SM (0 = uncapped) and
-// the join of the short-range stream before the solve.
+// the join of the short-range stream before the solve.  The FP64 path tries all
+// five.  In the mixed path registers cap the one-warp blocks at 8 an SM, two
+// warps a quarter, and fewer only lose (6 or 4 an SM: 7,580-7,596 us a call at
+// 32,000 waters against 7,516-7,551), so the join is all there is to choose; timings
+// of one and the same launch differ by some 7%, hence the repeats.
 struct ShortSched {
     int cap;
     bool join_before_solve;
 };
 constexpr int kNSched = 5;
 constexpr ShortSched kSched[kNSched] = {{3, false}, {0, false}, {2, false}, {0, true}, {3, true}};
-constexpr int kTuneWarm = 2, kTuneReps = 2;
-
+constexpr int kSchedFp64[kNSched] = {0, 1, 2, 3, 4}, kSchedMixed[2] = {1, 3};
+constexpr int kTuneWarm = 2;
+struct TunePlan {
+    const int *cand;   // places in kSched
+    int n, reps;       // timed evaluations of each
+};
+TunePlan tune_plan(const sibfa_ctx *ctx) {
+    if (ctx->prec == SIBFA_PREC_FP64) return {kSchedFp64, kNSched, 2};
+    return {kSchedMixed, 2, 4};
+}
 ShortSched short_sched(const sibfa_ctx *ctx) {
     const auto &T = ctx->tune;
-    if (!T.on) return {ctx->kp.periodic ? 3 : 0, false};
-    return kSched[T.choice >= 0 ? T.choice : T.cand];
+    if (!T.on) return {ctx->kp.periodic && ctx->prec == SIBFA_PREC_FP64 ? 3 : 0, false};
+    return kSched[T.choice >= 0 ? T.choice : tune_plan(ctx).cand[T.cand]];
 }
 int short_cap(const sibfa_ctx *ctx) { return short_sched(ctx).cap; }
-
 // Reads the last timed evaluation (waiting for it, only while tuning) and
 // advances the candidate; after the last candidate, fixes the fastest.
 void tune_account(sibfa_ctx *ctx) {
@@ -530,16 +542,17 @@ void tune_account(sibfa_ctx *ctx) {
         return;
     }
     if (T.seen++ < kTuneWarm) return;
-    T.tmin[T.cand] = std::min(T.tmin[T.cand], ms);
-    if (++T.reps < kTuneReps) return;
+    const TunePlan plan = tune_plan(ctx);
+    float &t = T.tmin[plan.cand[T.cand]];
+    t = std::min(t, ms);
+    if (++T.reps < plan.reps) return;
     T.reps = 0;
-    if (++T.cand < kNSched) return;
-    int best = 0;
-    for (int c = 1; c < kNSched; ++c)
-        if (T.tmin[c] < T.tmin[best]) best = c;
+    if (++T.cand < plan.n) return;
+    int best = plan.cand[0];
+    for (int k = 1; k < plan.n; ++k)
+        if (T.tmin[plan.cand[k]] < T.tmin[best]) best = plan.cand[k];
     T.choice = best;
 }
-
 sibfa_status join_rec(sibfa_ctx *ctx) {
     CK(cudaEventRecord(ctx->ev_join, ctx->s2));
     CK(cudaStreamWaitEvent(ctx->s, ctx->ev_join, 0));
@@ -930,8 +943,8 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
         ctx->short_pending = true;
         Phase ph(ctx, "short", ctx->s3);
         DevState<R> ds = short_view(d);
-        // resident blocks per SM (0: uncapped), chosen by the autotuner: a cap
-        // leaves every SM registers for the solve's small kernels
+        // resident blocks per SM (0: uncapped), chosen by the autotuner in FP64: a
+        // cap leaves every SM registers for the solve's small kernels
         launch_short(p, ds, Launch{ctx->s3, &ctx->launches}, short_cap(ctx));
     }
     // mixed periodic path: the FP64 intramolecular Ewald energy, beside everything else

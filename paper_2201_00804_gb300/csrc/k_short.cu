@@ -722,10 +722,9 @@ __global__ void __launch_bounds__(128) k_short_gather(KParams p, DevState<R> d, 
 
 }  // namespace
 
-template <typename R, bool PER>
+template <bool PER>
 static cudaError_t short_admit() {
-    constexpr int PART = sizeof(R) == 4 ? 2 : -1;
-    const auto k = k_short<R, PER, false, PART>;
+    const auto k = k_short<double, PER, false, -1>;
     int dev = 0, most = 0;
     cudaFuncAttributes fa;
     cudaError_t e = cudaGetDevice(&dev);
@@ -739,11 +738,14 @@ static cudaError_t short_admit() {
 // limit belongs to the process, so a launch that set its own could be refused
 // when another thread's context lowered it in between.
 template <typename R>
-cudaError_t short_init(const KParams &p) { return p.periodic ? short_admit<R, true>() : short_admit<R, false>(); }
+cudaError_t short_init(const KParams &p) {
+    if (sizeof(R) == 4) return cudaSuccess;
+    return p.periodic ? short_admit<true>() : short_admit<false>();
+}
 
-// max_per_sm > 0 caps the resident blocks per SM (FP32: warps, at four times
-// that) by reserving unused dynamic shared memory, which leaves registers on
-// every SM for the kernels of the other streams.
+// FP64: max_per_sm > 0 caps the resident blocks per SM by reserving unused
+// dynamic shared memory, which leaves registers on every SM for the kernels of
+// the other streams.  FP32 takes no cap (SHORT_BLOCKS an SM by its registers).
 template <typename R>
 void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm) {
     int dev = 0, per_sm = 0;
@@ -763,8 +765,8 @@ void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm) {
     const unsigned ng = (unsigned)((p.M + 3) / 4);
     auto run = [&](auto per, auto vir) {
         auto k = k_short<R, decltype(per)::value, decltype(vir)::value, PART>;
-        const int cap = sizeof(R) == 4 ? 4 * max_per_sm : max_per_sm;
-        if (cap > 0 && cap < SHORT_BLOCKS && !p.vir) {   // (registers allow no more than SHORT_BLOCKS)
+        const int cap = max_per_sm;
+        if (sizeof(R) == 8 && cap > 0 && cap < 8 && !p.vir) {   // (registers allow no more than 8)
             cudaFuncAttributes fa;
             cudaFuncGetAttributes(&fa, k);
             // one byte more per block than another block would leave room for
