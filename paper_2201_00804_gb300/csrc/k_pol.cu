@@ -558,7 +558,7 @@ constexpr int FM = 8;   // molecules per block
 template <typename R>
 struct FinIn {
     R G[FM][NP][3], mu[FM][NS][3], th[FM][NS][6], dv[FM][2][3];   // gradients, sensitivities, d V_lp
-    R ml[FM][NS * NMP], off[FM][NP][3], q[FM][NS], lam[FM][2], kap[FM][3];
+    R ml[FM][NS * NMP], off[FM][NP][3], q[FM][NS], lam[FM][2], kap[FM][3];   // kap: times ke
 };
 // A thread's elements of one array of PER values a molecule (stride apart)
 template <int PER, typename T = double>
@@ -575,6 +575,10 @@ struct FinLoad {
     __device__ __forceinline__ void add(const FinLoad &o) {
 #pragma unroll
         for (int k = 0; k < N; ++k) v[k] += o.v[k];
+    }
+    __device__ __forceinline__ void scale(T f) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[k] *= f;
     }
     template <typename R> __device__ __forceinline__ void put(R *out, int nm) const {
 #pragma unroll
@@ -601,6 +605,7 @@ __global__ void __launch_bounds__(128) k_finalize(KParams p, DevState<R> d, doub
     u.add(ur);
     h.add(hr);
     dv.add(dvr);
+    kap.scale(p.ke);   // rounded once
     g.put(&S.G[0][0][0], nm);
     u.put(&S.mu[0][0][0], nm);
     h.put(&S.th[0][0][0], nm);
@@ -683,7 +688,7 @@ __global__ void __launch_bounds__(128) k_finalize(KParams p, DevState<R> d, doub
             // charge-transfer dependence through the intramolecular potentials V_int(O, H1, H2)
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                const R kk = S.kap[l][a] * R(p.ke);
+                const R kk = S.kap[l][a];
                 if (kk == R(0)) continue;
 #pragma unroll
                 for (int s = 0; s < NS; ++s) {
