@@ -269,7 +269,7 @@ sibfa_status alloc_state(sibfa_ctx *ctx, DevState<R> &d) {
     AL(d.muR, M * 9);
     AL(d.lamR, M * 2);
     AL(d.tl_n, M * 3);
-    const size_t nt = (size_t)M * 3 * ctx->kp.tls;
+    const size_t nt = ctx->kp.tlist ? (size_t)M * 3 * ctx->kp.tls : 1;   // clusters that solve on their own keep no list
     AL(d.tl_j, nt);
     AL(d.tl_x, nt);
     AL(d.tl_y, nt);
@@ -1473,9 +1473,8 @@ sibfa_status sibfa_create(const sibfa_params *params, const sibfa_topology *topo
         ctx->kp.tls = 3 * nmax;
         // small gas-phase clusters of the mixed path: one block each, which
         // recomputes the products and needs no pair list
-        const char *e = getenv("SIBFA_PCG_HOST_LOOP");
-        if (e && e[0] == '1') ctx->pcg_graph_state = -1;
-        else if (!opts->periodic && opts->precision == SIBFA_PREC_MIXED && nmax + 1 <= CLUSTER_MAX) {
+        if (host_loop()) ctx->pcg_graph_state = -1;
+        else if (own_cluster_solve(opts->periodic, opts->precision, nmax + 1)) {
             ctx->cluster_max = nmax + 1;
             ctx->kp.tlist = 0;
         }

@@ -1,5 +1,6 @@
 // The polarization solve as one kernel: what the host lays out for it.
 #pragma once
+#include <cstdlib>
 #include <vector>
 
 #include "pcg_guess.cuh"
@@ -61,6 +62,16 @@ cudaError_t launch_pcg_loop(const KParams &p, DevState<R> &d, const LoopPlan &lp
 // Largest cluster the per-cluster solve takes (waters): its displacements,
 // n (n - 1) of them, stay in shared memory (48 KB at 64 waters).
 constexpr int CLUSTER_MAX = 64;
+// SIBFA_PCG_HOST_LOOP=1: solves are driven from the host, by separate kernels
+inline bool host_loop() {
+    const char *e = std::getenv("SIBFA_PCG_HOST_LOOP");
+    return e && e[0] == '1';
+}
+// Whether a context whose largest cluster has n waters solves each on its own,
+// and so records no pair list
+inline bool own_cluster_solve(int periodic, int precision, int n) {
+    return !host_loop() && !periodic && precision == SIBFA_PREC_MIXED && n <= CLUSTER_MAX;
+}
 // Admits the largest cluster's shared memory; once per context, at creation.
 cudaError_t cluster_init();
 // Every cluster of a gas-phase batch (mixed path) on its own, one block each; nmax: the largest.

@@ -27,6 +27,7 @@
 
 #include <cuda_runtime.h>
 
+#include "pcg_loop.cuh"
 #include "server_internal.h"
 
 namespace {
@@ -72,14 +73,16 @@ Shape shape_of(const sibfa_job &j) {
     return s;
 }
 
-// Device memory a context for the job needs: the polarization pair list, the
-// neighbour list and the short-range rows per molecule, the per-molecule state, the SPME grids and
+// Device memory a context for the job needs: the polarization pair list (none
+// where a cluster solves on its own), the neighbour list and the short-range
+// rows per molecule, the per-molecule state, the SPME grids and
 // a fixed allowance for the context and cuFFT.  An estimate with margin.
 size_t estimate_bytes(const sibfa_job &j, int precision) {
     const int nb = j.periodic ? 384 : std::max(1, std::min(384, j.n_mol - 1));
     const size_t entry = precision == SIBFA_PREC_FP64 ? 36 : 20;
+    const size_t list = sibfa::own_cluster_solve(j.periodic, precision, j.n_mol) ? 0 : (size_t)3 * 3 * nb * entry;
     const size_t per_mol =
-        (size_t)3 * 3 * nb * entry + (size_t)nb * (precision == SIBFA_PREC_FP64 ? 28 : 16) + 6144 +
+        list + (size_t)nb * (precision == SIBFA_PREC_FP64 ? 28 : 16) + 6144 +
         (j.periodic ? (size_t)192 * 16 : (size_t)nb * 24 * (precision == SIBFA_PREC_FP64 ? 2 : 1)) *
             (precision == SIBFA_PREC_FP64 ? 8 : 4);
     size_t b = (size_t)j.n_mol * per_mol;
