@@ -191,7 +191,11 @@ typedef struct sibfa_ctx sibfa_ctx;
  * solve; see sibfa_tuned_schedule) over its first full evaluations outside
  * sibfa_minimize by timing them and then keeps the fastest; the choice
  * affects scheduling only, never the results.  SIBFA_TUNE=0 at creation
- * turns the tuning off (fixed shape). */
+ * turns the tuning off (fixed shape).  SIBFA_MAX_DEVICE_BYTES=n at creation
+ * bounds the context's own device arrays (cuFFT's come on top): a box that is
+ * short of memory, under this bound or on the device, keeps fewer rows for its
+ * short-range gradients (same results, slower); what cannot fit is
+ * SIBFA_E_OOM. */
 sibfa_status sibfa_create(const sibfa_params *params, const sibfa_topology *topo,
                           const sibfa_run_opts *opts, sibfa_ctx **out);
 

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include <algorithm>
+#include <cstdint>
 #include <cstdlib>
 
 #include "sibfa_internal.cuh"
@@ -97,6 +98,7 @@ struct sibfa_ctx {
     std::string err = "no error";
     uint64_t launches = 0;
     size_t dev_bytes = 0;         // device memory allocated by the context
+    size_t dev_max = SIZE_MAX;    // and the most it may allocate
     int last_iters = 0;
     double last_resid = 0;
     double e_tail = 0;            // dispersion beyond rc (homogeneous fluid), added to disp and the virial
@@ -169,14 +171,15 @@ namespace {
 template <typename T>
 sibfa_status dalloc(sibfa_ctx *ctx, T **p, size_t n) {
     void *q = nullptr;
-    cudaError_t e = cudaMalloc(&q, n * sizeof(T) + 16);
+    const size_t bytes = n * sizeof(T) + 16;
+    cudaError_t e = bytes > ctx->dev_max - ctx->dev_bytes ? cudaErrorMemoryAllocation : cudaMalloc(&q, bytes);
     if (e != cudaSuccess) {
         ctx->err = std::string("cudaMalloc: ") + cudaGetErrorString(e);
         return SIBFA_E_OOM;
     }
-    cudaMemsetAsync(q, 0, n * sizeof(T) + 16, ctx->s);   // ordered before any later work on the stream
+    cudaMemsetAsync(q, 0, bytes, ctx->s);   // ordered before any later work on the stream
     ctx->allocs.push_back(q);
-    ctx->dev_bytes += n * sizeof(T) + 16;
+    ctx->dev_bytes += bytes;
     *p = (T *)q;
     return SIBFA_OK;
 }
@@ -237,10 +240,6 @@ sibfa_status alloc_state(sibfa_ctx *ctx, DevState<R> &d) {
     }
     AL(d.ctin, M * 8);
     AL(d.spk, M * 20);
-    // Inbox rows of the short-range pairs: in a box half the list's capacity (a molecule owns about half of its
-    // pairs; more rows than that are added directly), in the gas phase one a neighbour and part
-    d.in_rows = ctx->opts.periodic ? MAXN / 2 : (sizeof(R) == 4 ? 1 : 2) * (ctx->kp.tls / 3);
-    AL(d.inbox, (size_t)M * d.in_rows * (ctx->opts.periodic ? 16 : 24));
     AL(d.inn, M);
     AL(d.epart, M * NTERM);
     AL(d.epw, M * NS * 2);
@@ -1277,6 +1276,21 @@ sibfa_status create_impl(sibfa_ctx *ctx, const sibfa_topology *topo) {
         CKF(cufftSetStream(ctx->c2r2, ctx->s2));
         ctx->have_fft = true;
     }
+    // Inbox rows of the short-range pairs, after everything that a context
+    // cannot do without: in a box the method works with any number of them,
+    // so that a box that only just fits the device takes fewer; in the gas
+    // phase one a neighbour and part.
+    if (ctx->opts.periodic) {
+        d.in_rows = box_rows(ctx->opts.rc, M, ctx->opts.box);
+        while ((st = dalloc(ctx, &d.inbox, (size_t)M * d.in_rows * 16)) == SIBFA_E_OOM && d.in_rows > 0) {
+            cudaGetLastError();
+            d.in_rows /= 2;
+        }
+        if (st) return st;
+    } else {
+        d.in_rows = (sizeof(R) == 4 ? 1 : 2) * (ctx->kp.tls / 3);
+        AL(d.inbox, (size_t)M * d.in_rows * 24);
+    }
     CK(cudaStreamSynchronize(ctx->s));
     return SIBFA_OK;
 }
@@ -1480,8 +1494,9 @@ sibfa_status sibfa_create(const sibfa_params *params, const sibfa_topology *topo
         }
     }
     {
-        const char *t = getenv("SIBFA_TUNE");
+        const char *t = getenv("SIBFA_TUNE"), *b = getenv("SIBFA_MAX_DEVICE_BYTES");
         if (t && t[0] == '0') ctx->tune.on = false;
+        if (b && *b) ctx->dev_max = strtoull(b, nullptr, 10);
     }
     if (opts->periodic) {
         const double cell = opts->rc + 2.6 + LIST_SKIN;   // rc + 2 * maximum site extent (1.3 A) + skin

@@ -83,7 +83,7 @@ size_t estimate_bytes(const sibfa_job &j, int precision) {
     const size_t list = sibfa::own_cluster_solve(j.periodic, precision, j.n_mol) ? 0 : (size_t)3 * 3 * nb * entry;
     const size_t per_mol =
         list + (size_t)nb * (precision == SIBFA_PREC_FP64 ? 28 : 16) + 6144 +
-        (j.periodic ? (size_t)192 * 16 : (size_t)nb * 24 * (precision == SIBFA_PREC_FP64 ? 2 : 1)) *
+        (j.periodic ? (size_t)sibfa::box_rows(j.rc, j.n_mol, j.box) * 16 : (size_t)nb * 24 * (precision == SIBFA_PREC_FP64 ? 2 : 1)) *
             (precision == SIBFA_PREC_FP64 ? 8 : 4);
     size_t b = (size_t)j.n_mol * per_mol;
     if (j.periodic) b += (size_t)j.grid[0] * j.grid[1] * j.grid[2] * (precision == SIBFA_PREC_FP64 ? 80 : 44);

@@ -846,6 +846,15 @@ inline int warp_molecules(int M, double own, int parts, int per_sm, double margi
 }
 
 template <typename R> cudaError_t short_init(const KParams &p);
+// Inbox rows of a molecule in a box: half of its pairs, some 0.5 x the
+// neighbours within rc + 1.4 A at the box's density or, where that is lower (a
+// droplet, a slab), at that of water, 1.3 times over and 16 more for their
+// spread (rc 9: 119 rows of 16 values; half the list's capacity, 192, at most).
+// Further rows are added directly.
+inline int box_rows(double rc, int n_mol, const double box[3]) {
+    const double rn = rc + 1.4, rho = fmax(0.0334, n_mol / (box[0] * box[1] * box[2]));
+    return (int)fmin(MAXN / 2, ceil(0.65 * rho * 4.18879 * rn * rn * rn) + 16.0);
+}
 template <typename R> void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm = 0);
 template <typename R> void launch_ct(const KParams &p, DevState<R> &d, Launch L);
 template <typename R> void launch_intra_perm(const KParams &p, DevState<R> &d, Launch L);

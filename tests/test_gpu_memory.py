@@ -63,3 +63,41 @@ def test_admission_does_not_charge_a_list_that_is_not_kept():
         assert r["status"] == 0
     finally:
         srv.close()
+
+
+@pytest.mark.parametrize("prec,tol", [("PREC_FP64", 1e-9), ("PREC_MIXED", 2e-5)])
+def test_box_that_only_just_fits(prec, tol, monkeypatch):
+    """A context that may not have all the memory it would take keeps fewer rows
+    for the short-range gradients, down to none, and gives the same forces (to the
+    bounds of FP64, with the solve at 1e-12, and of FP32, of the largest)."""
+    import paper_2201_00804_gb300 as pkg
+    s, o = synth.make_config("water216")
+    pos = np.ascontiguousarray(s.pos.reshape(-1))
+    kw = dict(periodic=True, box=s.box, rc=o["rc"], grid=o["grid"], ewald_alpha=o["ewald"],
+              pcg_tol_D=1e-12 if prec == "PREC_FP64" else 1e-7, precision=getattr(pkg, prec), warm_start=False)
+
+    def run():
+        ctx = pkg.sibfa_create(synth.PARAMS, s.mp_local, **kw)
+        F = np.zeros_like(pos)
+        try:
+            return pkg.sibfa_energy_forces(ctx, pos, F), F
+        finally:
+            pkg.sibfa_destroy(ctx)
+
+    e0, F0 = run()
+    rows = 216 * 70 * 16 * (8 if prec == "PREC_FP64" else 4)   # bytes of all rows at rc 7
+    lo, hi = 1 << 20, 1 << 26   # the least bound under which creation succeeds
+    while hi - lo > 4096:
+        mid = (lo + hi) // 2
+        monkeypatch.setenv("SIBFA_MAX_DEVICE_BYTES", str(mid))
+        try:
+            pkg.sibfa_destroy(pkg.sibfa_create(synth.PARAMS, s.mp_local, **kw))
+            hi = mid
+        except pkg.SibfaError:
+            lo = mid
+    for bound in (hi, hi + rows // 4, hi + rows // 2, hi + rows):
+        monkeypatch.setenv("SIBFA_MAX_DEVICE_BYTES", str(bound))
+        e1, F1 = run()
+        for t in ("rep", "disp", "xdisp"):
+            assert abs(e0[t] - e1[t]) <= tol * abs(e0[t]), (bound, t)
+        assert np.abs(F0 - F1).max() <= tol * np.abs(F0).max(), bound
