@@ -256,6 +256,12 @@ sibfa_status sibfa_cluster_terms(sibfa_ctx *ctx, sibfa_energy_terms *terms);
  * (cuFFT executions are not counted). */
 uint64_t sibfa_kernel_launches(const sibfa_ctx *ctx);
 
+/* How often a block of the polarization solve's cooperative kernel polls the
+ * others' counter before it gives up and the call returns SIBFA_E_TIMEOUT
+ * (2^22 unless set, some seconds; 0: every wait gives up at once, which is how
+ * a test makes one run out).  The next call starts from the direct field. */
+void sibfa_set_wait_polls(sibfa_ctx *ctx, unsigned polls);
+
 /* Launch shape of the short-range kernels chosen by the context's tuning:
  * *blocks_per_sm = resident blocks per SM (0 = uncapped, as always on the
  * mixed path), *done = 1 once the

@@ -26,5 +26,6 @@ from .sibfa import (  # noqa: F401
     sibfa_profile_clear,
     sibfa_profile_get,
     sibfa_set_profiling,
+    sibfa_set_wait_polls,
     sibfa_solve_dipoles,
 )

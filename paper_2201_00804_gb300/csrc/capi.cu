@@ -851,9 +851,11 @@ sibfa_status evaluate_graph(sibfa_ctx *ctx, bool want_forces, bool dipoles_only,
             return SIBFA_OK;
         }
         ctx->capturing = true;
+        const bool had_mu = ctx->have_mu;
         const sibfa_status a = evaluate_impl<R>(ctx, want_forces, dipoles_only, tol);
         const sibfa_status b = join_short(ctx), c = join_ct(ctx);
         ctx->capturing = false;
+        ctx->have_mu = had_mu;   // nothing has run yet
         const cudaError_t e = cudaStreamEndCapture(ctx->s, &graph);
         g->launches = ctx->launches - before;
         ctx->launches = before;
@@ -1040,6 +1042,11 @@ sibfa_status evaluate_impl(sibfa_ctx *ctx, bool want_forces, bool dipoles_only, 
 }
 
 sibfa_status check_flags(sibfa_ctx *ctx, int flags) {
+    if (flags & F_TIMEOUT) {   // an abandoned solve leaves nothing to start the next one from
+        ctx->have_mu = false;
+        ctx->hist_n = 0;
+        ctx->md_forces_valid = false;
+    }
     if (flags & F_CUTOFF) {
         ctx->err = "cutoff plus twice the site extent exceeds half the box (or a site is > 1.3 A from its O)";
         return SIBFA_E_CUTOFF;
@@ -1685,6 +1692,12 @@ void sibfa_profile_clear(sibfa_ctx *ctx) {
         ctx->event_pool.push_back(s.b);
     }
     ctx->spans.clear();
+}
+
+void sibfa_set_wait_polls(sibfa_ctx *ctx, unsigned polls) {
+    if (!ctx) return;
+    ctx->loop.polls = polls;
+    drop_eval_graphs(ctx);
 }
 
 uint64_t sibfa_kernel_launches(const sibfa_ctx *ctx) { return ctx ? ctx->launches : 0; }

@@ -35,8 +35,6 @@ namespace {
 constexpr int LT = 512;          // threads per block
 constexpr int LREC = 256;        // of them on the reciprocal chain (periodic)
 constexpr int PGL = 8;           // lanes per atom in the gather
-// polls of the grid counter before a block gives up (seconds; the waits are microseconds)
-constexpr unsigned BAR_POLLS = 1u << 22;
 
 template <typename R> struct Cplx;
 template <> struct Cplx<float> { using T = float2; };
@@ -390,11 +388,11 @@ __device__ inline void take_row(const R *row, int K2, int zb, const R *w, R &t0,
 // Arrival at and wait for the grid-wide counter, one thread per block.  A
 // wait that runs out raises the shared give-up flag, and every block then
 // leaves at its next barrier.
-__device__ __noinline__ bool counter_wait(unsigned *bar, unsigned target) {
+__device__ __noinline__ bool counter_wait(unsigned *bar, unsigned target, unsigned polls) {
     __threadfence();
     atomicAdd(bar, 1u);
     unsigned v;
-    for (unsigned k = 0; k < BAR_POLLS; ++k) {
+    for (unsigned k = 0; k < polls; ++k) {
         asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
         if (v >= target) return true;
         if ((k & 1023u) == 1023u && *(volatile unsigned *)(bar + 1)) return false;
@@ -588,13 +586,13 @@ __global__ void __launch_bounds__(LT, 2)
     auto everyone = [&]() {
         __syncthreads();
         target += ncta;
-        if (tid == 0 && !counter_wait(bar, target)) s_lost = 1;
+        if (tid == 0 && !counter_wait(bar, target, lp.polls)) s_lost = 1;
         __syncthreads();
     };
     auto chain = [&]() {
         part_sync<LREC>();
         target += ncta;
-        if (tid == 0 && !counter_wait(bar, target)) s_lost = 1;
+        if (tid == 0 && !counter_wait(bar, target, lp.polls)) s_lost = 1;
         part_sync<LREC>();
     };
 

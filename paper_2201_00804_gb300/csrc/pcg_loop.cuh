@@ -33,6 +33,7 @@ struct LoopPlan {
     int ncta = 0;                    // blocks (0: this context's solves take the separate kernels)
     int mper = 0;                    // molecules per block
     int maxit = 200;
+    unsigned polls = 1u << 22;       // of the grid counter before a block gives up (seconds; the waits are microseconds)
     FftAxis ax[3] = {};
     int ntw = 0;                     // twiddles of all axes
     int xt = 0;                      // (ky, kz) columns per tile of the x transforms

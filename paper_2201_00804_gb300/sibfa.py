@@ -121,6 +121,8 @@ def load_library(path: str = LIB_PATH):
     lib.sibfa_tuned_schedule.argtypes = [C.c_void_p, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int),
                                          C.POINTER(C.c_double), C.c_int]
     lib.sibfa_tuned_schedule.restype = C.c_int
+    lib.sibfa_set_wait_polls.argtypes = [C.c_void_p, C.c_uint]
+    lib.sibfa_set_wait_polls.restype = None
     lib.sibfa_set_profiling.argtypes = [C.c_void_p, C.c_int]
     lib.sibfa_set_profiling.restype = None
     lib.sibfa_profile_get.argtypes = [C.c_void_p, C.c_char_p, C.POINTER(C.c_double), C.POINTER(C.c_int)]
@@ -369,6 +371,11 @@ def sibfa_tuned_shape(ctx):
     st = lib.sibfa_tuned_shape(ctx, C.byref(b), C.byref(dn))
     _check(lib, ctx, st)
     return b.value, bool(dn.value)
+
+
+def sibfa_set_wait_polls(ctx, polls: int):
+    """Polls before a wait of the one-kernel solve gives up (SIBFA_E_TIMEOUT); 0: at once."""
+    load_library().sibfa_set_wait_polls(ctx, int(polls))
 
 
 def sibfa_set_profiling(ctx, on):
