@@ -246,6 +246,7 @@ sibfa_status alloc_state(sibfa_ctx *ctx, DevState<R> &d) {
     AL(d.vir, M * 9);
     AL(d.vir_r, M * 9);
     AL(d.vir_s, M * 9);
+    AL(d.vir_w, ctx->opts.periodic ? 1 : (size_t)M * NS * 2 * 9);
     AL(d.vphi, M * 9);
     AL(d.gpt_r, M * NP * 3);
     AL(d.gpt_s, M * NP * 3);

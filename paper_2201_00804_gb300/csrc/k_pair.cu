@@ -3,7 +3,7 @@
 // Every kernel walks the neighbours of one molecule i and accumulates only
 // i's quantities (energy halves, gradients of i's points, multipole
 // sensitivities of i's sites), so no two threads write the same output and
-// no atomics are needed (k_perm_gas: two warps add to a target); the neighbour list is full, each molecule pair is
+// no atomics are needed (k_perm_gas: two warps add to a target, once each); the neighbour list is full, each molecule pair is
 // visited from both sides.  Pair arithmetic runs in R (float in the mixed
 // path, double in the FP64 path); per-lane partial sums are reduced across
 // the warp in double.
@@ -467,6 +467,7 @@ __global__ void __launch_bounds__(32, sizeof(R) == 4 ? GAS_BLOCKS : 8) k_perm_ga
     const int lane = threadIdx.x, w = blockIdx.y;
     const bool energy = blockIdx.z == 0;
     GasWalk walk(p, d, mpw, lane);
+    double carry = 0.0;
     for (bool fresh = true; fresh = walk.at == 0, walk.next(lane);) {
         PermAcc<R> acc;
         acc.gr = mk(R(0), R(0), R(0));
@@ -518,7 +519,12 @@ __global__ void __launch_bounds__(32, sizeof(R) == 4 ? GAS_BLOCKS : 8) k_perm_ga
         __syncwarp();
         const double ke = p.ke;
         walk.segments(fresh, [&](int m, int c0, int c1, bool first) {
-            const double t = segment_sum<R>(buf, lane, NV, c0, c1);
+            double t = segment_sum<R>(buf, lane, NV, c0, c1);
+            if (!first) t += carry;
+            if (c1 == walk.n_used && walk.at != 0) {   // goes on in the next round
+                carry = t;
+                return;
+            }
             double *dst = nullptr;
             if (lane < 3) dst = d.gpt + (m * NP + w) * 3 + lane;
             else if (lane < 6) dst = d.gmu + (m * NS + w) * 3 + lane - 3;
@@ -527,12 +533,10 @@ __global__ void __launch_bounds__(32, sizeof(R) == 4 ? GAS_BLOCKS : 8) k_perm_ga
             if (dst) atomicAdd(dst, (lane < 6 ? ke : (lane < 12 ? ke * (1.0 / 3.0) : 1.0)) * t);
             // per-site energies (summed over the five sites in a fixed order by k_pol_energy)
             const double e = ke * (t + __shfl_down_sync(0xffffffffu, t, 1));
-            if (energy && (lane == 15 || lane == 17)) {
-                double *o = d.epw + (m * NS + w) * 2 + (lane == 17);
-                *o = first ? e : *o + e;
-            }
-            if (VIR && lane >= 19 && lane < NV) atomicAdd(d.vir + m * 9 + lane - 19, ke * t);
-            if (energy && w < 3 && lane == 0 && first) d.tl_n[m * 3 + w] = 3 * d.nnbr[m];
+            if (energy && (lane == 15 || lane == 17)) d.epw[(m * NS + w) * 2 + (lane == 17)] = e;
+            // and the virials of the sites' two sides
+            if (VIR && lane >= 19 && lane < NV) d.vir_w[(((size_t)m * NS + w) * 2 + blockIdx.z) * 9 + lane - 19] = ke * t;
+            if (energy && w < 3 && lane == 0) d.tl_n[m * 3 + w] = 3 * d.nnbr[m];
         });
         __syncwarp();
     }

@@ -511,6 +511,12 @@ __global__ void k_pol_energy(KParams p, DevState<R> d) {
     for (int w = 0; w < NS; ++w) el += d.epw[(m * NS + w) * 2], pe += d.epw[(m * NS + w) * 2 + 1];
     d.epart[m * NTERM + T_ELEC] += el;
     d.epart[m * NTERM + T_PEN] += pe;
+    if (p.vir && !p.periodic)   // and in the gas phase the virials of the sites' two sides
+        for (int k = 0; k < 9; ++k) {
+            double v = 0;
+            for (int s = 0; s < 2 * NS; ++s) v += d.vir_w[((size_t)m * 2 * NS + s) * 9 + k];
+            d.vir[m * 9 + k] += v;
+        }
 }
 template <typename R>
 void launch_pol_energy(const KParams &p, DevState<R> &d, Launch L) {

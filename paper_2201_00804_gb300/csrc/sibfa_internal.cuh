@@ -190,6 +190,7 @@ struct DevState {
     double *vir;        // M*9
     double *vir_r;      // M*9 (reciprocal chain)
     double *vir_s;      // M*9 (short-range kernels)
+    double *vir_w;      // M*NS*2*9 (gas phase: permanent pass, by site and side)
     double *virk;       // 2 passes x VK_BLOCKS x 8: k-space sums per convolution block
     void *qhat_p;       // K0*K1*(K2/2+1) complex: spectrum of the permanent grid (kept for the force pass)
     R *vphi;            // M*9 gradient of the reciprocal permanent potential at O, H1, H2
