@@ -464,6 +464,8 @@ __global__ void __launch_bounds__(32, sizeof(R) == 4 ? SHORT_BLOCKS : 8) k_short
     __shared__ R qd[3][64];   // queued pairs: molecules and displacement
     constexpr int NV = PER ? (VIR ? 24 : 15) : 1;
     __shared__ R buf[NV * 33];   // a box: column sums of molecule cur, by lane
+    constexpr bool FOLD = PER && sizeof(R) == 4;   // energies go on in FP64 from molecule to molecule
+    __shared__ double es[FOLD ? 3 : 1][32];
     const int lane = threadIdx.x;
     const int part = PART < 0 ? (int)blockIdx.y : PART;
     const Scal<R> &S = sc<R>(p);
@@ -471,6 +473,7 @@ __global__ void __launch_bounds__(32, sizeof(R) == 4 ? SHORT_BLOCKS : 8) k_short
     const int first = blockIdx.x * mpw, last = min(p.M, first + mpw);
     Acc<R> Er, Ed, Ex;
     int cur = -1;
+    if constexpr (FOLD) es[0][lane] = es[1][lane] = es[2][lane] = 0.0;
     auto store = [&]() {   // points 3, 4 are the lone pairs (point slots 5, 6)
         __syncwarp();
         if (lane < NV) {
@@ -536,6 +539,7 @@ __global__ void __launch_bounds__(32, sizeof(R) == 4 ? SHORT_BLOCKS : 8) k_short
             }
         }
         // into the sums of its molecule, one molecule at a time in order
+        bool begun = false;
         while (PER) {
             if (cur >= 0 && mi == cur) {
 #pragma unroll
@@ -558,7 +562,20 @@ __global__ void __launch_bounds__(32, sizeof(R) == 4 ? SHORT_BLOCKS : 8) k_short
             if (cur >= 0) store();
             clear();
             cur = next;
+            begun = true;
         }
+        if constexpr (FOLD) {
+            if (begun) {   // (each lane its own places)
+                es[0][lane] += Er.get();
+                es[1][lane] += Ed.get();
+                es[2][lane] += Ex.get();
+                Er = Ed = Ex = Acc<R>();
+            }
+        }
+    };
+    auto total = [&](const Acc<R> &a, int k) {
+        if constexpr (FOLD) return warp_sum(es[k][lane] + a.get());
+        else return warp_sum_acc(a);
     };
     int nq = 0;
     for (int i = first; i < last; ++i) {
@@ -643,7 +660,7 @@ __global__ void __launch_bounds__(32, sizeof(R) == 4 ? SHORT_BLOCKS : 8) k_short
     if (PER) {
         if (cur >= 0) store();
         // the energies are summed over all molecules of the box
-        const double e0 = warp_sum_acc(Er), e1 = warp_sum_acc(Ed), e2 = warp_sum_acc(Ex);
+        const double e0 = total(Er, 0), e1 = total(Ed, 1), e2 = total(Ex, 2);
         if (lane == 0) {
             double *e = d.epart + first * NTERM;
             if (part != 1) atomicAdd(e + T_REP, e0);
