@@ -925,6 +925,7 @@ __global__ void __launch_bounds__(CT, 8)
     k_pcg_cluster(KParams p, DevState<float> d, int maxit, MuGuess guess, int warm, double *push) {
     __shared__ double sh[2][CT];
     __shared__ double s_sum[2], s_val[2];
+    __shared__ float s_top;
     const int tid = threadIdx.x;
     const int m0 = d.cl_start[blockIdx.x], n = d.cl_start[blockIdx.x + 1] - m0, n3 = n * 3, n9 = n * 9;
     double *mu = reinterpret_cast<double *>(loop_raw), *r = mu + n9, *pv = r + n9, *ap = pv + n9;
@@ -1006,6 +1007,12 @@ __global__ void __launch_bounds__(CT, 8)
     double rz = s_sum[0];
     int it = 0;
     bool done = s_sum[1] < tol2;
+    // Thread EST follows the Lanczos matrix of the iteration (diagonal 1/a_k +
+    // beta_(k-1)/a_(k-1), beside it sqrt(beta_k)/a_k), whose row sums bound the
+    // eigenvalues of 1 - alpha T that the residual has met.
+    constexpr int EST = 32;
+    float ia = 0.f, below = 0.f, side = 0.f, top = 0.f;
+    if (tid == EST) s_top = 1e30f;   // no iteration: nothing known
     while (!done && it < maxit) {
         field();
         double v1[1] = {0};
@@ -1016,6 +1023,7 @@ __global__ void __launch_bounds__(CT, 8)
         }
         block_totals<1>(v1, sh, s_sum, tid);
         if (tid == 0) s_val[0] = rz / s_sum[0];
+        if (tid == EST) ia = (float)s_sum[0] / (float)rz;
         __syncthreads();
         const double a = s_val[0];
         v2[0] = v2[1] = 0;
@@ -1028,6 +1036,13 @@ __global__ void __launch_bounds__(CT, 8)
         }
         block_totals<2>(v2, sh, s_sum, tid);
         if (tid == 0) s_val[1] = s_sum[0] / rz;
+        if (tid == EST) {
+            const float b = (float)s_sum[0] / (float)rz, e = sqrtf(b) * ia;
+            top = fmaxf(top, ia + below + side + e);
+            below = b * ia;
+            side = e;
+            s_top = top;
+        }
         __syncthreads();
         const double beta = s_val[1];
         rz = s_sum[0];
@@ -1041,9 +1056,13 @@ __global__ void __launch_bounds__(CT, 8)
     }
     // The last residual is at hand: one more Jacobi step costs no product and
     // leaves the dipoles closer (the batch used to iterate until its slowest
-    // cluster was done, which over-converged the others).
+    // cluster was done, which over-converged the others).  It multiplies the
+    // residual by alpha T, and so is left out unless the eigenvalues met lie below
+    // 2: waters at liquid distances stay below 1.5, but pressed together to O-O
+    // distances near 1 A some pass 3, and the step would lead away from the tolerance.
+    const bool closer = s_top < 2.f;
     for (int e = tid; e < n9; e += CT) {
-        const double m = mu[e] + p.a_pol[(e / 3) % 3] * r[e];
+        const double m = closer ? mu[e] + p.a_pol[(e / 3) % 3] * r[e] : mu[e];
         d.mu[m0 * 9 + e] = m;
         if (push) push[m0 * 9 + e] = m;
     }
