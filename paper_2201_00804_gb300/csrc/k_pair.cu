@@ -334,7 +334,7 @@ __device__ __forceinline__ double segment_sum(const R *buf, int lane, int nv, in
 // the pipe of each quarter of an SM, few, which spreads the work (824 waters: 510 us at 4, 570 at 8, 802 at 16).
 template <typename R>
 int gas_mpw(const KParams &p) {
-    return warp_molecules(p.M, 0.5 * (p.M / (double)p.n_cl - 1.0), 2 * NS, (sizeof(R) == 4 ? GAS_BLOCKS : 4), 0.25,
+    return warp_molecules(p.M, 0.5 * (p.M / (double)p.n_cl - 1.0), 0.5 * (p.tls / 3), 2 * NS, (sizeof(R) == 4 ? GAS_BLOCKS : 4), 0.25,
                           sizeof(R) == 4 ? 32 : 4);
 }
 

@@ -776,7 +776,9 @@ void launch_short(const KParams &p, DevState<R> &d, Launch L, int max_per_sm) {
     // between the O).
     const double rn = p.rc + 1.4, V = p.box[0] * p.box[1] * p.box[2];
     const double nbr = p.periodic ? std::min(p.M - 1.0, p.M / V * 4.18879 * rn * rn * rn) : p.M / (double)p.n_cl - 1.0;
-    const int mpw = warp_molecules(p.M, 0.5 * nbr, parts, sizeof(R) == 4 ? SHORT_BLOCKS : 4, p.periodic ? 0.0 : 0.25, 64);
+    const double most = p.periodic ? nbr : (double)(p.tls / 3);
+    const int mpw = warp_molecules(p.M, 0.5 * nbr, 0.5 * most, parts, sizeof(R) == 4 ? SHORT_BLOCKS : 4,
+                                   p.periodic ? 0.0 : 0.25, 64);
     size_t sm = 0;
     k_short_pack<R><<<(p.M * 5 + 255) / 256, 256, 0, L.s>>>(p, d);
     const unsigned ng = (unsigned)((p.M + 3) / 4);

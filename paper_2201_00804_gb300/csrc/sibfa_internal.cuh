@@ -831,16 +831,20 @@ template <typename R> void launch_real_perm(const KParams &p, DevState<R> &d, La
 template <typename R> void launch_lp_potential(const KParams &p, DevState<R> &d, Launch L);
 // Molecules that a one-warp block takes, of which each has `own` entries of
 // work, so that `parts` such grids need the fewest rounds of 32 entries in a
-// row over the blocks that the device holds at once (per_sm an SM).  margin:
-// part of a round for molecules that have more than the average.
-inline int warp_molecules(int M, double own, int parts, int per_sm, double margin, int most) {
+// row over the blocks that the device holds at once (per_sm an SM).  own_max:
+// entries of a molecule of the largest cluster, of which a block may get nothing
+// else; such a block may take twice as long as the rest (one cluster of 385
+// beside 5,000 of 1: 1427 us a call with the mean alone, now 688; 4,096 clusters of
+// 2-32: 2831 us where such a block counts in full, now 2757).  margin: part of a
+// round for molecules that have more than the average.
+inline int warp_molecules(int M, double own, double own_max, int parts, int per_sm, double margin, int most) {
     int dev = 0, n_sm = 0, k_best = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     double best = 1e30;
     for (int k = 1; k <= most; ++k) {
         const double waves = ceil((double)((M + k - 1) / k) * parts / ((double)n_sm * per_sm));
-        const double c = waves * ceil(margin + k * (own > 0.5 ? own : 0.5) / 32.0);
+        const double c = fmax(waves * ceil(margin + k * (own > 0.5 ? own : 0.5) / 32.0), 0.5 * ceil(k * own_max / 32.0));
         if (c < best) best = c, k_best = k;
     }
     return k_best;
