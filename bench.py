@@ -839,10 +839,11 @@ def main():
     api = make_api()
     F_host = torch.zeros(M * 9, dtype=torch.float64).pin_memory()
     hosts = [snap.cpu().pin_memory() for snap in snapshots]
-    # untimed: the new context's schedule tuning (its first full evaluations)
+    # untimed: warm-up calls (a small context replays its evaluations from the
+    # third on), and the new context's schedule tuning where it has one
     for k in range(32):
         pkg.sibfa_energy_forces(api, hosts[k % len(hosts)], F_host)
-        if pkg.sibfa_tuned_shape(api)[1]:
+        if k >= 3 and pkg.sibfa_tuned_shape(api)[1]:
             break
     pkg.sibfa_energy_forces(api, hosts[0], F_host)
     e2e_s = 0.0

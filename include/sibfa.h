@@ -184,9 +184,13 @@ typedef struct sibfa_ctx sibfa_ctx;
  * some 1700 waters, on a grid whose axes are products of 2, 3 and 5, as one
  * cooperative kernel, for gas-phase clusters of up to 64 waters on the mixed
  * path as one block per cluster (each cluster stops on its own residual),
- * otherwise as a CUDA graph with a conditional while-node.  With the environment variable SIBFA_PCG_HOST_LOOP=1 at
- * creation it is driven from the host instead (one launch per kernel and
- * iteration), which kernel profilers can follow.  The context tunes the schedule of its short-range kernels
+ * otherwise as a CUDA graph with a conditional while-node.  With the
+ * environment variable SIBFA_PCG_HOST_LOOP=1 at creation it is driven from the
+ * host instead, by separate kernels (one launch per kernel and iteration), which
+ * kernel profilers can follow; for the systems of the one-kernel solves these
+ * are other kernels, with another form of the recurrence, the FFT library's
+ * transforms and no replayed evaluations.  An FP64 context tunes the schedule
+ * of its short-range kernels
  * (resident blocks per SM, and whether they finish before the polarization
  * solve; see sibfa_tuned_schedule) over its first full evaluations outside
  * sibfa_minimize by timing them and then keeps the fastest; the choice
@@ -271,8 +275,8 @@ sibfa_status sibfa_tuned_shape(const sibfa_ctx *ctx, int *blocks_per_sm, int *do
 
 /* The whole short-range schedule chosen by the tuning.  The candidates, in
  * order: (blocks per SM, joined before the solve) = (3, no), (0, no),
- * (2, no), (0, yes), (3, yes), on the mixed path only the two without a
- * cap; "joined before the solve" means the
+ * (2, no), (0, yes), (3, yes); the mixed path has (0, no) only and times
+ * nothing.  "Joined before the solve" means the
  * short-range kernels finish before the polarization solve starts (the
  * solve's latency-bound kernels then have the SMs to themselves), otherwise
  * they run beside it until the chain rule.  *blocks_per_sm, *join_before_solve

@@ -35,19 +35,18 @@ struct sibfa_ctx {
     cudaStream_t s3 = nullptr;
     cudaEvent_t ev_fork3 = nullptr, ev_join3 = nullptr;
     bool short_pending = false;
-    // Autotuner of the short-range schedule: resident blocks per SM (FP64 path;
-    // 0 = uncapped) and whether the short-range stream is joined before the
+    // Autotuner of the FP64 path's short-range schedule: resident blocks per SM
+    // (0 = uncapped) and whether the short-range stream is joined before the
     // polarization solve (the solve then has the SMs to itself) or only
     // before the chain rule.  The first evaluations outside sibfa_minimize
     // after two warm-up ones
     // each run one candidate and are timed whole on the main stream (two per
-    // candidate in FP64, four in the mixed path, the fastest kept); then the
-    // fastest candidate is fixed.  The choice changes only the scheduling, never
-    // the arithmetic.
+    // candidate, the faster kept); then the fastest candidate is fixed.  The
+    // choice changes only the scheduling, never the arithmetic.
     struct ShortTuner {
         bool on = true;
         int seen = 0;            // evaluations with forces seen
-        int cand = 0;            // candidate being timed (place in the precision's list)
+        int cand = 0;            // candidate being timed
         int reps = 0;
         int choice = -1;         // fixed candidate, -1 while tuning
         float tmin[5] = {1e30f, 1e30f, 1e30f, 1e30f, 1e30f};
@@ -501,32 +500,25 @@ sibfa_status join_ct(sibfa_ctx *ctx) {
     return SIBFA_OK;
 }
 
-// Short-range schedule candidates: resident blocks per SM (0 = uncapped) and
-// the join of the short-range stream before the solve.  The FP64 path tries all
-// five.  In the mixed path registers cap the one-warp blocks at 8 an SM, two
-// warps a quarter, and fewer only lose (6 or 4 an SM: 7,580-7,596 us a call at
-// 32,000 waters against 7,516-7,551), so the join is all there is to choose; timings
-// of one and the same launch differ by some 7%, hence the repeats.
+// Short-range schedule candidates of the FP64 path: resident blocks per SM (0 =
+// uncapped) and the join of the short-range stream before the solve.  The mixed
+// path has one schedule and times nothing: its one-warp blocks are capped at 8 an
+// SM by their registers, and fewer only lose (6 or 4 an SM: 7,580-7,596 us a call at
+// 32,000 waters against 7,516-7,551); the join was slower wherever it was timed (8
+// waters 118 us against 107, 216: 510 and 498, 2,600: 1090 and 1000, 4,096: 1425 and 1350, 32,000:
+// 7420 and 7290, 4,096 clusters 2745 and 2665; MD of 216 to 17,576 waters 1 to 10%,
+// of 32,000 within 1% either way).
 struct ShortSched {
     int cap;
     bool join_before_solve;
 };
 constexpr int kNSched = 5;
 constexpr ShortSched kSched[kNSched] = {{3, false}, {0, false}, {2, false}, {0, true}, {3, true}};
-constexpr int kSchedFp64[kNSched] = {0, 1, 2, 3, 4}, kSchedMixed[2] = {1, 3};
-constexpr int kTuneWarm = 2;
-struct TunePlan {
-    const int *cand;   // places in kSched
-    int n, reps;       // timed evaluations of each
-};
-TunePlan tune_plan(const sibfa_ctx *ctx) {
-    if (ctx->prec == SIBFA_PREC_FP64) return {kSchedFp64, kNSched, 2};
-    return {kSchedMixed, 2, 4};
-}
+constexpr int kTuneWarm = 2, kTuneReps = 2;
 ShortSched short_sched(const sibfa_ctx *ctx) {
     const auto &T = ctx->tune;
     if (!T.on) return {ctx->kp.periodic && ctx->prec == SIBFA_PREC_FP64 ? 3 : 0, false};
-    return kSched[T.choice >= 0 ? T.choice : tune_plan(ctx).cand[T.cand]];
+    return kSched[T.choice >= 0 ? T.choice : T.cand];
 }
 int short_cap(const sibfa_ctx *ctx) { return short_sched(ctx).cap; }
 // Reads the last timed evaluation (waiting for it, only while tuning) and
@@ -542,15 +534,13 @@ void tune_account(sibfa_ctx *ctx) {
         return;
     }
     if (T.seen++ < kTuneWarm) return;
-    const TunePlan plan = tune_plan(ctx);
-    float &t = T.tmin[plan.cand[T.cand]];
-    t = std::min(t, ms);
-    if (++T.reps < plan.reps) return;
+    T.tmin[T.cand] = std::min(T.tmin[T.cand], ms);
+    if (++T.reps < kTuneReps) return;
     T.reps = 0;
-    if (++T.cand < plan.n) return;
-    int best = plan.cand[0];
-    for (int k = 1; k < plan.n; ++k)
-        if (T.tmin[plan.cand[k]] < T.tmin[best]) best = plan.cand[k];
+    if (++T.cand < kNSched) return;
+    int best = 0;
+    for (int c = 1; c < kNSched; ++c)
+        if (T.tmin[c] < T.tmin[best]) best = c;
     T.choice = best;
 }
 sibfa_status join_rec(sibfa_ctx *ctx) {
@@ -1503,7 +1493,7 @@ sibfa_status sibfa_create(const sibfa_params *params, const sibfa_topology *topo
     }
     {
         const char *t = getenv("SIBFA_TUNE"), *b = getenv("SIBFA_MAX_DEVICE_BYTES");
-        if (t && t[0] == '0') ctx->tune.on = false;
+        if ((t && t[0] == '0') || opts->precision == SIBFA_PREC_MIXED) ctx->tune.on = false;
         if (b && *b) ctx->dev_max = strtoull(b, nullptr, 10);
     }
     if (opts->periodic) {

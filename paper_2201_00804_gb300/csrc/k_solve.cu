@@ -1023,7 +1023,7 @@ __global__ void __launch_bounds__(CT, 8)
         }
         block_totals<1>(v1, sh, s_sum, tid);
         if (tid == 0) s_val[0] = rz / s_sum[0];
-        if (tid == EST) ia = (float)s_sum[0] / (float)rz;
+        if (tid == EST) ia = __fdividef((float)s_sum[0], (float)rz);
         __syncthreads();
         const double a = s_val[0];
         v2[0] = v2[1] = 0;
@@ -1037,7 +1037,7 @@ __global__ void __launch_bounds__(CT, 8)
         block_totals<2>(v2, sh, s_sum, tid);
         if (tid == 0) s_val[1] = s_sum[0] / rz;
         if (tid == EST) {
-            const float b = (float)s_sum[0] / (float)rz, e = sqrtf(b) * ia;
+            const float b = __fdividef((float)s_sum[0], (float)rz), e = __fsqrt_rn(b) * ia;
             top = fmaxf(top, ia + below + side + e);
             below = b * ia;
             side = e;

@@ -354,8 +354,8 @@ def sibfa_kernel_launches(ctx) -> int:
 
 def sibfa_tuned_schedule(ctx):
     """(short-range blocks per SM, joined before the solve, True once tuning
-    fixed it, the five candidates' fastest timed evaluations in ms, 0 for
-    one not tried: on the mixed path only the two without a cap are)."""
+    fixed it, the five candidates' fastest timed evaluations in ms, 0 where
+    not timed: the mixed path has one schedule and times none)."""
     lib = load_library()
     b, j, dn = C.c_int(), C.c_int(), C.c_int()
     ms = (C.c_double * 5)()

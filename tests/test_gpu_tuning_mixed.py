@@ -1,5 +1,6 @@
-"""The schedule tuning of the mixed path.  Its short-range kernel takes no cap
-on the blocks per SM, so there are two schedules to try, and no cap to report."""
+"""The mixed path has one schedule of its short-range kernel (its registers cap
+the blocks per SM already, and finishing it before the solve only loses), so
+there is nothing to time and no cap to report, from the first call on."""
 import numpy as np
 import pytest
 
@@ -18,7 +19,7 @@ def _lib():
 
 
 @pytest.mark.parametrize("periodic", [True, False], ids=["box", "gas"])
-def test_two_schedules_and_no_cap(periodic, monkeypatch):
+def test_one_schedule_and_no_cap(periodic):
     import paper_2201_00804_gb300 as pkg
     if periodic:
         s, o = synth.make_config("water216")
@@ -28,18 +29,9 @@ def test_two_schedules_and_no_cap(periodic, monkeypatch):
     pos = np.ascontiguousarray(s.pos.reshape(-1))
     ctx = pkg.sibfa_create(synth.PARAMS, s.mp_local, precision=pkg.PREC_MIXED, warm_start=False, **kw)
     try:
-        assert pkg.sibfa_tuned_shape(ctx) == (0, False)
-        for _ in range(11):   # 2 warm-up + 2 schedules x 4 timed, each read at the next call
+        for _ in range(16):
+            assert pkg.sibfa_tuned_shape(ctx) == (0, True)
+            assert pkg.sibfa_tuned_schedule(ctx) == (0, False, True, [0.0] * 5)
             pkg.sibfa_energy_forces(ctx, pos)
-        blocks, join, done, ms = pkg.sibfa_tuned_schedule(ctx)
-        assert done and blocks == 0 and pkg.sibfa_tuned_shape(ctx) == (0, True)
-        assert [t > 0 for t in ms] == [False, True, False, True, False]
-        assert join == (ms[3] < ms[1])
-    finally:
-        pkg.sibfa_destroy(ctx)
-    monkeypatch.setenv("SIBFA_TUNE", "0")
-    ctx = pkg.sibfa_create(synth.PARAMS, s.mp_local, precision=pkg.PREC_MIXED, warm_start=False, **kw)
-    try:
-        assert pkg.sibfa_tuned_schedule(ctx)[:3] == (0, False, True)
     finally:
         pkg.sibfa_destroy(ctx)
