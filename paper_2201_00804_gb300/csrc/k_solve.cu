@@ -1011,7 +1011,7 @@ __global__ void __launch_bounds__(CT, 8)
     // beta_(k-1)/a_(k-1), beside it sqrt(beta_k)/a_k), whose row sums bound the
     // eigenvalues of 1 - alpha T that the residual has met.
     constexpr int EST = 32;
-    float ia = 0.f, below = 0.f, side = 0.f, top = 0.f;
+    float frz = (float)rz, ia = 0.f, below = 0.f, side = 0.f, top = 0.f;
     if (tid == EST) s_top = 1e30f;   // no iteration: nothing known
     while (!done && it < maxit) {
         field();
@@ -1023,7 +1023,7 @@ __global__ void __launch_bounds__(CT, 8)
         }
         block_totals<1>(v1, sh, s_sum, tid);
         if (tid == 0) s_val[0] = rz / s_sum[0];
-        if (tid == EST) ia = __fdividef((float)s_sum[0], (float)rz);
+        if (tid == EST) ia = __fdividef((float)s_sum[0], frz);
         __syncthreads();
         const double a = s_val[0];
         v2[0] = v2[1] = 0;
@@ -1037,7 +1037,8 @@ __global__ void __launch_bounds__(CT, 8)
         block_totals<2>(v2, sh, s_sum, tid);
         if (tid == 0) s_val[1] = s_sum[0] / rz;
         if (tid == EST) {
-            const float b = __fdividef((float)s_sum[0], (float)rz), e = __fsqrt_rn(b) * ia;
+            const float f = (float)s_sum[0], b = __fdividef(f, frz), e = b * rsqrtf(fmaxf(b, 1e-30f)) * ia;
+            frz = f;
             top = fmaxf(top, ia + below + side + e);
             below = b * ia;
             side = e;
