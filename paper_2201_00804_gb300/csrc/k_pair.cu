@@ -330,8 +330,8 @@ __device__ __forceinline__ double segment_sum(const R *buf, int lane, int nv, in
     return sizeof(R) == 4 ? a.get() : double(s);
 }
 // Molecules a warp of k_perm_gas: whole rounds in FP32 (4096 clusters of 17
-// waters: 1318 us at 2, 1234 at 4, 1154 at 8, 1113 at 32); in FP64, bound by
-// the pipe of each quarter of an SM, few, which spreads the work (824 waters: 510 us at 4, 570 at 8, 802 at 16).
+// waters, at most 2: 1305 us, 4: 1351, 8: 1135, 32: 1050); in FP64, bound by
+// the pipe of each quarter of an SM, few, which spreads the work (824 waters, at most 2 or 4: 510 us, 8: 522, 16: 703).
 template <typename R>
 int gas_mpw(const KParams &p) {
     return warp_molecules(p.M, 0.5 * (p.M / (double)p.n_cl - 1.0), 0.5 * (p.tls / 3), 2 * NS, (sizeof(R) == 4 ? GAS_BLOCKS : 4), 0.25,
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(VIR ? 32 * NS : 32,
 // energy, a quarter of the work here (see perm_pair), is the same from both
 // sides of a pair: it is taken from the entries that own their pair (blockIdx.z
 // = 0), and the others skip it.  Bound by issue and latency at 16 warps an SM (127
-// registers; 14: 1152 us).  4096 clusters of 17 waters 1282 -> 1113 us, 824
+// registers).  4096 clusters of 17 waters 1282 -> 1050 us, 824
 // waters in FP64 clusters 600 -> 510 us, against a warp per target site with queues.
 template <typename R, bool VIR>
 __global__ void __launch_bounds__(32, sizeof(R) == 4 ? GAS_BLOCKS : 8) k_perm_gas(KParams p, DevState<R> d, int mpw) {

@@ -21,12 +21,13 @@
 //
 // Bound in FP32 by the latency of one lane's long chains at two warps a
 // quarter of an SM (255 registers, no spill; issue slots 55% busy): with 10,
-// 12 and 16 blocks an SM, at 200, 168 and 128 registers, 32,000 waters (rc 9) took
-// 996, 992 and 1132 us against 923 (before rows were written as vectors).  In FP64 bound by the FP64
-// pipe; repulsion and dispersion go to different warps, which fills the chip better.
+// 12 and 16 blocks an SM, at 168, 168 and 128 registers with spills, 32,000 waters (rc 9) took
+// 914, 912 and 1126 us against 762.  In FP64 bound by the FP64
+// pipe (255 registers, 1.9 to 2.1 KB a thread spilled); repulsion and dispersion go to different warps,
+// which fills the chip better.
 // All launches together, before (item queues) and now: 32,000 waters 1815 and
-// 745 us, 4,096 waters 279 and 130, 4,096 clusters of 17 waters 930 and 408, 216 waters in FP64
-// 486 and 265, 824 waters in FP64 clusters 592 and 230.
+// 762 us, 4,096 waters 279 and 135, 4,096 clusters of 17 waters 930 and 408, 216 waters in FP64
+// 486 and 266, 824 waters in FP64 clusters 592 and 232.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
